@@ -401,7 +401,7 @@ mbis_status mbis::create_ctx(const mbis_event* ev, const double* psd, const mbis
   }
   CREATE_TRY(dalloc(c, &c->d_err, sizeof(int32_t)));
   CREATE_TRY(cudaMemsetAsync(c->d_err, 0, sizeof(int32_t), s));
-  CREATE_TRY(dalloc(c, &c->red.partials, sizeof(double) * 2 * kReduceBlocks));
+  CREATE_TRY(dalloc(c, &c->red.partials, sizeof(double) * 3 * kReduceBlocks));
   CREATE_TRY(dalloc(c, &c->red.counter, sizeof(unsigned int)));
   CREATE_TRY(cudaMemsetAsync(c->red.counter, 0, sizeof(unsigned int), s));
   CREATE_TRY(dalloc(c, &c->red.result, sizeof(double) * 4));
@@ -483,7 +483,7 @@ size_t mbis::ctx_footprint_bytes(int32_t n_det, int32_t n_bins, int32_t dtype, c
   size_t t = 0;
   t += round_alloc((dtype == MBIS_C128 ? 16 : 8) * nb) + round_alloc(8 * nb);  // strain, PSD
   t += round_alloc(8 * kNumBasis * n) + round_alloc(8 * kGLSize) + round_alloc(4);
-  t += round_alloc(16 * kReduceBlocks) + round_alloc(4) + round_alloc(32);
+  t += round_alloc(24 * kReduceBlocks) + round_alloc(4) + round_alloc(32);
   t += round_alloc(8 * (size_t)moments_partials_size(kMaxP)) + round_alloc(4) + round_alloc(8 * kMomentSums);
   const size_t rows = fold ? 1 : nd;
   t += round_alloc(16 * n * rows) + round_alloc(8 * (n + 1) * rows) + round_alloc(8 * n * rows);  // C, T, scratch

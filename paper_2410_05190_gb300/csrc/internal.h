@@ -181,7 +181,7 @@ int32_t batch_ctas_per_sm(int32_t tile);
 
 // two-pass weight reduction; partials / counter / result are device scratch
 struct ReduceScratch {
-  double* partials;       // [2 * kReduceBlocks]
+  double* partials;       // [3 * kReduceBlocks]: (m_b, S1_b, S2_b) per CTA
   unsigned int* counter;  // [1], zero between calls
   double* result;         // [4]: m, s1, s2, n
 };

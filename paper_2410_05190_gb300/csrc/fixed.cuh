@@ -1,0 +1,154 @@
+// fixed.cuh -- fixed-point helpers of the double-precision kernels (host and device).
+//
+// The GB300 runs an FP64 instruction in 64 clocks per warp and SM quarter, a 32 x 32 + 64-bit
+// integer multiply-add in 2 (measured: 64.7 and 2.06).  Quantities whose magnitude is bounded
+// -- a phase in turns, a sine or cosine, data scaled by their largest value -- therefore keep
+// FP64 accuracy and better as 64-bit integers split into two 28-bit halves,
+//   X = X1 2^28 + X0,  0 <= X0 < 2^28,
+// a product of which takes three multiply-adds:
+//   A B = A1 B1 2^56 + (A1 B0 + A0 B1) 2^28 + (A0 B0, dropped: 2^-56 of the result's scale).
+// "Unit 2^-56" below means a 64-bit integer holding the value times 2^56.
+#pragma once
+#include <cstdint>
+#include <cstring>
+
+#include "physics.cuh"
+
+namespace mbis {
+
+struct Pair28 {
+  int32_t h, l;
+};
+
+MBIS_HD Pair28 pair28(int64_t x) { return Pair28{(int32_t)(x >> 28), (int32_t)((uint32_t)x & 0x0fffffffu)}; }
+
+// a b + c in 64 bits.  In PTX on the device: from the C++ expression the compiler made a 64 x
+// 64-bit product (3.5 multiply-adds) of halves that it could see being cut from 64-bit values.
+MBIS_HD int64_t madw(int32_t a, int32_t b, int64_t c) {
+#ifdef __CUDA_ARCH__
+  int64_t d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+#else
+  return (int64_t)a * (int64_t)b + c;
+#endif
+}
+MBIS_HD int64_t mulw(int32_t a, int32_t b) {
+#ifdef __CUDA_ARCH__
+  int64_t d;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+  return d;
+#else
+  return (int64_t)a * (int64_t)b;
+#endif
+}
+
+// (high word of a b), unsigned
+MBIS_HD uint32_t mulhi_u(uint32_t a, uint32_t b) {
+#ifdef __CUDA_ARCH__
+  return __umulhi(a, b);
+#else
+  return (uint32_t)(((uint64_t)a * (uint64_t)b) >> 32);
+#endif
+}
+
+// a b + c with a, b in unit 2^-56 halves: unit 2^-56
+MBIS_HD int64_t mul28(Pair28 a, Pair28 b, int64_t c) {
+  const int64_t mid = madw(a.h, b.l, mulw(a.l, b.h));
+  return madw(a.h, b.h, c + (mid >> 28));
+}
+
+MBIS_HD uint64_t double_bits(double x) {
+#ifdef __CUDA_ARCH__
+  return (uint64_t)__double_as_longlong(x);
+#else
+  uint64_t b;
+  std::memcpy(&b, &x, 8);
+  return b;
+#endif
+}
+
+// exponent of the smallest power of two above |x| (|x| < 2^e), from the bits; 1025 for
+// infinities and NaN; zeros and subnormals count as 2^-1022
+MBIS_HD int32_t exponent_above(double x) { return (int32_t)((double_bits(x) >> 52) & 0x7ff) - 1022; }
+
+// round(x 2^e) as a 64-bit integer, by shifts (no FP64 arithmetic); |x 2^e| < 2^62
+MBIS_HD int64_t to_fixed(double x, int32_t e) {
+  const uint64_t b = double_bits(x);
+  const int32_t be = (int32_t)((b >> 52) & 0x7ff);
+  const int64_t m = be == 0 ? 0 : (int64_t)((b & 0xfffffffffffffull) | 0x10000000000000ull);  // x = m 2^(be - 1075)
+  const int32_t s = be - 1075 + e;
+  int64_t v;
+  if (s >= 0)
+    v = m << (s < 10 ? s : 10);
+  else
+    v = s < -54 ? 0 : (m + ((int64_t)1 << (-s - 1))) >> (-s);
+  return (b >> 63) ? -v : v;
+}
+
+// ---- sine and cosine of a phase in turns ------------------------------------------------
+// The phase P counts 2^-64 turns.  Its nearest multiple of 1/128 turn is i / 128 + q / 4
+// (i = 0..31, a table entry; q the quadrant), the rest r 2^-64 turns with |r| <= 2^56.  With
+// eta = r 2^-56 and zeta = eta^2 the Taylor series of the rest's angle rho = 2 pi 2^-8 eta are
+//   sin rho     = eta (A0 - zeta (A1 - zeta (A2 - zeta A3))),  A_m = (2 pi 2^-8)^(2m+1) / (2m+1)!
+//   cos rho - 1 = -zeta (B1 - zeta (B2 - zeta B3)),            B_m = (2 pi 2^-8)^(2m) / (2m)!
+// (the first terms left out are below 2^-60), evaluated in integers; the sum formulas with the
+// table entry and the quadrant give the phase's sine and cosine in unit 2^-56 with an
+// absolute error of a few 2^-56.
+struct TrigCell {
+  int32_t i, q;  // table entry, quadrant
+  Pair28 eta;    // unit 2^-56
+};
+
+MBIS_HD TrigCell trig_cell(uint64_t P) {
+  const uint64_t pr = P + (1ull << 56);
+  TrigCell c;
+  const uint32_t hi = (uint32_t)(pr >> 32), lo = (uint32_t)pr;
+  c.i = (int32_t)((hi >> 25) & 31);
+  c.q = (int32_t)(hi >> 30);
+  const int32_t rh = (int32_t)(hi & 0x01ffffffu) - 0x01000000;
+  c.eta.h = (int32_t)(((uint32_t)rh << 4) | (lo >> 28));
+  c.eta.l = (int32_t)(lo & 0x0fffffffu);
+  return c;
+}
+
+// 2^56 times the coefficients (B2, B3, A2, A3: in the units of the mulhi chains)
+constexpr double kRho = kTwoPi / 256.0;
+constexpr double kTwo56 = 72057594037927936.0, kTwo57 = 2.0 * kTwo56, kTwo58 = 2.0 * kTwo57;
+constexpr int64_t kTrigA0 = (int64_t)(kRho * kTwo56 + 0.5);
+constexpr int64_t kTrigA1 = (int64_t)(kRho * kRho * kRho / 6.0 * kTwo56 + 0.5);
+constexpr uint32_t kTrigA2 = (uint32_t)(kRho * kRho * kRho * kRho * kRho / 120.0 * kTwo57 + 0.5);
+constexpr uint32_t kTrigA3 = (uint32_t)(kRho * kRho * kRho * kRho * kRho * kRho * kRho / 5040.0 * kTwo58 + 0.5);
+constexpr int64_t kTrigB1 = (int64_t)(kRho * kRho / 2.0 * kTwo56 + 0.5);
+constexpr uint32_t kTrigB2 = (uint32_t)(kRho * kRho * kRho * kRho / 24.0 * kTwo57 + 0.5);
+constexpr uint32_t kTrigB3 = (uint32_t)(kRho * kRho * kRho * kRho * kRho * kRho / 720.0 * kTwo58 + 0.5);
+
+// cosine and sine of the cell's phase from the table entry's (tc, ts), unit 2^-56 halves
+MBIS_HD void trig_eval(const TrigCell& c, Pair28 tc, Pair28 ts, int64_t& cos_out, int64_t& sin_out) {
+  // zeta = eta^2, unit 2^-56, and its leading 31 bits
+  const int64_t z64 = madw(c.eta.h, c.eta.h, mulw(c.eta.h, c.eta.l) >> 27);
+  const Pair28 z = pair28(z64);
+  const uint32_t x = (uint32_t)((uint64_t)z64 >> 25);  // unit 2^-31
+  // x (unit 2^-31) times a unit 2^-57 factor: the high word has unit 2^-56
+  const int64_t u = kTrigB1 - (int64_t)mulhi_u(x, kTrigB2 - mulhi_u(x, kTrigB3));
+  const int64_t s = kTrigA1 - (int64_t)mulhi_u(x, kTrigA2 - mulhi_u(x, kTrigA3));
+  const int64_t cm = -mul28(z, pair28(u), 0);          // cos rho - 1
+  const int64_t v = kTrigA0 - mul28(z, pair28(s), 0);
+  const int64_t sn = mul28(c.eta, pair28(v), 0);       // sin rho
+  const Pair28 m = pair28(cm), n = pair28(sn);
+  const int64_t tc64 = ((int64_t)tc.h << 28) + tc.l, ts64 = ((int64_t)ts.h << 28) + ts.l;
+  // cos = tc + tc cm - ts sn, sin = ts + ts cm + tc sn
+  int64_t mc = madw(tc.h, m.l, mulw(tc.l, m.h));
+  mc = madw(-ts.h, n.l, madw(-ts.l, n.h, mc));
+  int64_t ms = madw(ts.h, m.l, mulw(ts.l, m.h));
+  ms = madw(tc.h, n.l, madw(tc.l, n.h, ms));
+  const int64_t co = madw(tc.h, m.h, madw(-ts.h, n.h, tc64 + (mc >> 28)));
+  const int64_t si = madw(ts.h, m.h, madw(tc.h, n.h, ts64 + (ms >> 28)));
+  // the quadrant: (cos, sin) -> (-sin, cos) per quarter turn (negation to 2^-56: ~x = -x - 1)
+  const bool odd = c.q & 1;
+  const int64_t c0 = odd ? si : co, s0 = odd ? co : si;
+  cos_out = c0 ^ -(int64_t)(((c.q + 1) >> 1) & 1);
+  sin_out = s0 ^ -(int64_t)(c.q >> 1);
+}
+
+}  // namespace mbis

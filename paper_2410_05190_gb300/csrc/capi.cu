@@ -49,6 +49,19 @@ double q_integral(double a, double b) {
   return s;
 }
 
+// scratch of split folded launches of up to n samples
+cudaError_t split_scratch(mbis_ctx* c, int32_t parts, int64_t n) {
+  dfree(c, c->d_zpart);
+  dfree(c, c->d_amp);
+  dfree(c, c->d_kcut);
+  c->split_cap = 0;
+  cudaError_t e = dalloc(c, &c->d_zpart, sizeof(double2) * (size_t)parts * (size_t)n);
+  if (e == cudaSuccess) e = dalloc(c, &c->d_amp, sizeof(double) * (size_t)n);
+  if (e == cudaSuccess) e = dalloc(c, &c->d_kcut, sizeof(int32_t) * (size_t)n);
+  if (e == cudaSuccess) c->split_cap = n;
+  return e;
+}
+
 void free_tables(mbis_ctx* c) {
   dfree(c, c->d_cfold64);
   dfree(c, c->d_tfold);
@@ -746,38 +759,28 @@ mbis_status mbis_loglike(mbis_ctx* c, int64_t n, const double* theta, double* lo
     if (!a.fold)
       return fail(c, MBIS_E_UNSUPPORTED,
                   "mbis_loglike: mixed precision with sampled sky/orientation needs MBIS_MARG_TIME");
-    // a launch with fewer tiles than the device has CTA slots splits each tile's bins over
-    // several CTAs (whole parts each), so small batches still fill the GPU
+    // A launch of up to four waves of tiles gives each tile one CTA per part of its bins: the
+    // GPU stays full to the end, at the price of a repeated set-up (~0.1 of a part's time) and
+    // of the epilogue.  Measured on 16-part grids (ms, whole tiles -> one-part pieces):
+    // 10^4 samples 0.90, 2^17 7.9 (both always split); 2*10^5 13.0 -> 11.9, 2^18 16.3 -> 15.5,
+    // 4*10^5 24.0 -> 23.5; two-part pieces lose (2^16: 4.18 against 4.10).
     LikeArgs b = a;
-    const int64_t tiles = (n + kMixedThreads - 1) / kMixedThreads, slots = (int64_t)c->n_sms * 8;
+    const int64_t tiles = (n + kMixedThreads - 1) / kMixedThreads, slots = (int64_t)c->n_sms * kFoldCtasPerSm;
     const int32_t parts = (c->n_bins + kPartBins - 1) / kPartBins;
-    // the split minimises waves x (parts per piece + the set-up, ~0.1 of a part's time): a
-    // 2^16-sample batch (512 tiles, 16 parts) runs 16 one-part pieces in 6.7 waves rather
-    // than 2 eight-part pieces in a wave 84% full
-    b.split = 1;
-    if (tiles < slots && parts > 1) {
-      double best = 1e300;
-      for (int32_t sp = 1; sp <= parts; ++sp) {
-        const double waves = std::ceil((double)(tiles * sp) / (double)slots);
-        const double t = waves * (std::ceil((double)parts / sp) + 0.1);
-        if (t < best) {
-          best = t;
-          b.split = sp;
-        }
+    b.split = parts > 1 && tiles < 4 * slots ? parts : 1;
+    if (b.split > 1 && tiles >= slots && c->split_cap < n) {
+      // beyond one wave the scratch (16 bytes per sample and part) only buys speed: whole tiles
+      // when it cannot be had, or while the stream is being captured
+      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+      CU_TRY(c, cudaStreamIsCapturing(s, &cap));
+      if (cap != cudaStreamCaptureStatusNone || split_scratch(c, parts, n) != cudaSuccess) {
+        (void)cudaGetLastError();
+        b.split = 1;
       }
     }
     if (const mbis_status r = sample_order(c, a, kFoldOrderGran, s, &b.perm); r != MBIS_OK) return r;
     if (b.split > 1) {
-      if (c->split_cap < n) {
-        dfree(c, c->d_zpart);
-        dfree(c, c->d_amp);
-        dfree(c, c->d_kcut);
-        c->split_cap = 0;
-        CU_TRY(c, dalloc(c, &c->d_zpart, sizeof(double2) * (size_t)parts * (size_t)n));
-        CU_TRY(c, dalloc(c, &c->d_amp, sizeof(double) * (size_t)n));
-        CU_TRY(c, dalloc(c, &c->d_kcut, sizeof(int32_t) * (size_t)n));
-        c->split_cap = n;
-      }
+      if (c->split_cap < n) CU_TRY(c, split_scratch(c, parts, n));
       b.zpart = c->d_zpart;
       b.amp_out = c->d_amp;
       b.kcut_out = c->d_kcut;

@@ -30,6 +30,7 @@ constexpr int kChunk = 512;         // bins per shared-memory chunk of the mixed
 constexpr int kPartChunks = 16;
 constexpr int kPartBins = kPartChunks * kChunk;
 constexpr int kMixedThreads = 128;  // samples per CTA of the mixed kernel
+constexpr int kFoldCtasPerSm = 7;   // resident CTAs per SM of the single-event launch
 constexpr int kBatchCtasPerSm = 7;  // resident CTAs per SM of the persistent multi-event launch
 constexpr int kReduceBlocks = 608;  // 4 x 152 SMs
 constexpr int kReduceThreads = 256;

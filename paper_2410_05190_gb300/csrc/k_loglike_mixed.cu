@@ -146,8 +146,11 @@ __device__ __forceinline__ double fold_loglike(const LikeArgs& a, double A, int3
 // already run a tile (persistent launch): the mbarriers are then invalidated and initialised
 // afresh.  piece / split: this CTA sums the parts [n_parts piece / split, n_parts (piece + 1)
 // / split) of the tile's bins; with split > 1 it writes their sums for the epilogue kernel.
-// A sample's arithmetic does not depend on T or on its tile-mates.
-template <bool kFF, int T>
+// A sample's arithmetic does not depend on T or on its tile-mates.  U: bin pairs per trip of the
+// inner loop.  The persistent launch gains from 8 (its step on eight uneven events: 14.16 ms
+// at 1, 13.58 at 2, 12.84 at 3, 12.54 at 4, 12.44 at 8); the single-event launch, at 0.89 of
+// the sine/cosine rate, loses (2^20 BNS samples: 60.6 ms at 1, 64.0 at 2, 61.4 at 8).
+template <bool kFF, int T, int U = 1>
 __device__ __forceinline__ void fold_tile(const LikeArgs& a, int64_t tile, bool first, FoldSmem<T>& sm, int piece = 0,
                                           int split = 1) {
   float4 (&sC)[kNbuf][kChunk / 2] = sm.sC;
@@ -294,7 +297,7 @@ __device__ __forceinline__ void fold_tile(const LikeArgs& a, int64_t tile, bool 
         float2 w = make_float2(st.w, st.w + 1.0f);
         const int32_t npair = (my_end - k) >> 1;
         const float4* cp = cb + ((k - kb) >> 1);
-#pragma unroll 1
+#pragma unroll U
         for (int32_t p = 0; p < npair; ++p) {
           float2 R = cr[kFoldRemDeg];
 #pragma unroll
@@ -415,8 +418,10 @@ __global__ void fold_epilogue_kernel(LikeArgs a) {
   a.out[s] = fold_loglike(a, A, a.kcut_out[s], Zr, Zi);
 }
 
+// Seven CTAs per SM: at eight (64 registers) the sine/cosine pipe is no fuller (2^20 BNS
+// samples: 61.3 ms against 60.6; 2^16 samples of 8033 bins: 188 us against 181).
 template <bool kFF>
-__global__ void __launch_bounds__(kMixedThreads, 8) loglike_mixed_fold_kernel(LikeArgs a) {
+__global__ void __launch_bounds__(kMixedThreads, kFoldCtasPerSm) loglike_mixed_fold_kernel(LikeArgs a) {
   __shared__ FoldSmem<kMixedThreads> sm;
   const int split = a.split > 1 ? a.split : 1;
   fold_tile<kFF, kMixedThreads>(a, blockIdx.x / split, true, sm, (int)(blockIdx.x % split), split);
@@ -429,6 +434,8 @@ __global__ void __launch_bounds__(kMixedThreads, 8) loglike_mixed_fold_kernel(Li
 // Tiles of T samples with at most C CTAs per SM (the autotuner picks among (64, 14),
 // (128, 7) and (256, 3)): 72-85 registers hold the persistent loop's state without the
 // spills that a 64-register bound caused (6% faster on the uneven batch at T = 128).
+constexpr int kBatchUnroll = 8;
+
 template <bool kFF, int T, int C>
 __global__ void __launch_bounds__(T, C) loglike_mixed_batch_kernel(const LikeArgs* __restrict__ args,
                                                                    const BatchItem* __restrict__ items, int32_t n_items,
@@ -443,7 +450,7 @@ __global__ void __launch_bounds__(T, C) loglike_mixed_batch_kernel(const LikeArg
     __syncthreads();
     if (it >= n_items) break;
     const BatchItem item = items[it];
-    fold_tile<kFF, T>(args[item.ev], item.tile, first, sm);
+    fold_tile<kFF, T, kBatchUnroll>(args[item.ev], item.tile, first, sm);
     first = false;
     __syncthreads();
   }

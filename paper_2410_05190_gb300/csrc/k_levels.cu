@@ -13,6 +13,7 @@
 
 #include <cmath>
 
+#include "fpkey.cuh"
 #include "internal.h"
 
 namespace mbis {
@@ -26,16 +27,6 @@ constexpr int kMaxLevelSlots = 16;
 struct LevelRef {
   double r[kMaxLevelSlots];
 };
-
-// Comparisons on the integer pipe: an FP64 instruction holds its quarter of the SM for 64
-// clocks.  The key orders as the numbers do, with one zero; NaN has no key.
-__device__ __forceinline__ long long order_key(double x) {
-  const long long b = __double_as_longlong(x);
-  return b >= 0 ? b : (long long)(0x8000000000000000ull - (unsigned long long)b);
-}
-__device__ __forceinline__ bool is_nan(double x) {
-  return (unsigned long long)(__double_as_longlong(x) & 0x7fffffffffffffffll) > 0x7ff0000000000000ull;
-}
 
 __global__ void __launch_bounds__(kLevelThreads) levels_kernel(int64_t n, const double* __restrict__ theta,
                                                                const double* __restrict__ w, LevelRef ref,

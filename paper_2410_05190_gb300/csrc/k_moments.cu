@@ -14,6 +14,7 @@
 // through shared memory; per-CTA partials go to device scratch and the last CTA folds them
 // in a fixed order with all its threads.  Measured on a GB300 (device time, 5 slots): 83 us
 // at 2^18 samples and 48 us at 2^16 before, 26 and 14 us now.
+#include "fpkey.cuh"
 #include "internal.h"
 
 namespace mbis {
@@ -24,13 +25,6 @@ constexpr int kMomBlocks = 152;  // one per SM: the fold's cost grows with the w
 constexpr int kMomWarps = kMomThreads / 32;
 
 __host__ __device__ constexpr int moment_sums(int P) { return 1 + P + P * (P + 1) / 2; }
-
-// The order of FP64 numbers on the integer pipe (NaN apart): an FP64 comparison holds its
-// quarter of the SM for 64 clocks.
-__device__ __forceinline__ long long order_key(double x) {
-  const long long b = __double_as_longlong(x);
-  return b >= 0 ? b : (long long)(0x8000000000000000ull - (unsigned long long)b);
-}
 
 // Folds v[0 .. M) over the warp.  Afterwards lane l holds the total of sum `first` (and of
 // no other) for the lanes with first < M; every M up to 32 lanes' worth per call of the

@@ -3,109 +3,108 @@
 // longest among its lanes), while a sample's result does not depend on which CTA or lanes
 // it shares -- its bins past its own ISCO cut add exact zeros -- so ordering the samples by
 // their live bins only removes the work a CTA would spend on its longest sample.
-#include <algorithm>
-
 #include "internal.h"
+#include "order.cuh"
 
 namespace mbis {
 namespace {
 
-// live bins of sample i in units of gran bins (rounded up), estimated in FP32: the estimate
-// only steers the order; each CTA still runs to the exact cut of its samples
-__device__ __forceinline__ int32_t order_key(const LikeArgs& a, int64_t i, int32_t gran) {
-  const double mc = a.pos[kMc] >= 0 ? a.theta[(int64_t)a.pos[kMc] * a.n + i] : a.fixed[kMc];
-  const double q = a.pos[kQ] >= 0 ? a.theta[(int64_t)a.pos[kQ] * a.n + i] : a.fixed[kQ];
-  if (!(mc > 0.0) || !(q > 0.0)) return 0;
-  const float qf = (float)q;
-  const float m_sec = (float)(mc * kTsun) * powf(1.0f + qf, 1.2f) * powf(qf, -0.6f);
-  const float fi = 1.0f / (46.172139f * m_sec);  // 6^(3/2) pi M
-  const float k = fminf(fmaxf(ceilf((fi - (float)a.f_lo) / (float)a.df), 0.0f), (float)a.n_bins);
-  return ((int32_t)k + gran - 1) / gran;
-}
-
-// warp-uniform loop over the samples; lanes with the same key add once per warp
-__global__ void order_hist_kernel(LikeArgs a, int32_t gran, int32_t* hist) {
-  const int lane = threadIdx.x & 31;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < a.n; base += stride) {
-    const int64_t i = base + lane;
-    const bool on = i < a.n;
-    const unsigned mask = __ballot_sync(0xffffffffu, on);
-    if (on) {
-      const int32_t key = order_key(a, i, gran);
-      const unsigned peers = __match_any_sync(mask, key);
-      if (lane == __ffs(peers) - 1) atomicAdd(&hist[key], __popc(peers));
-    }
+// The part of LikeArgs that the key needs: a kernel's parameters are copied at each launch.
+struct BandKey {
+  const double *mc, *q;  // null: fixed
+  double mc0, q0;
+  float f_lo, df, n_bins;
+  int32_t gran;
+  // live bins of sample i in units of gran bins (rounded up), estimated in FP32: the estimate
+  // only steers the order; each CTA still runs to the exact cut of its samples
+  __device__ __forceinline__ int32_t operator()(int64_t i) const {
+    const float m = (float)(mc ? mc[i] : mc0), qf = (float)(q ? q[i] : q0);
+    if (!(m > 0.0f) || !(qf > 0.0f)) return 0;
+    const float m_sec = m * (float)kTsun * powf(1.0f + qf, 1.2f) * powf(qf, -0.6f);
+    const float fi = 1.0f / (46.172139f * m_sec);  // 6^(3/2) pi M
+    const float k = fminf(fmaxf(ceilf((fi - f_lo) / df), 0.0f), n_bins);
+    return ((int32_t)k + gran - 1) / gran;
   }
-}
+};
 
-// one CTA: counts -> first slot of each key, keys in decreasing order
-__global__ void order_scan_kernel(int32_t n_keys, int32_t* hist) {
+// one CTA: counts -> first slot of each key, keys in decreasing order.  Every thread owns a
+// contiguous run of keys, read and written as a whole; long key ranges (a bin pair per key on
+// a 128k-bin grid) go through shared memory in coalesced pieces.
+constexpr int kScanThreads = 1024;
+constexpr int kScanPer = 8;
+
+__global__ void __launch_bounds__(kScanThreads) order_scan_kernel(int32_t n_keys, int32_t* hist) {
   __shared__ int32_t warp_tot[32];
+  __shared__ int32_t piece[kScanThreads * (kScanPer + 1)];  // padded: a thread's run is conflict-free
+  __shared__ int32_t s_carry;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int per = (n_keys + (int)blockDim.x - 1) / (int)blockDim.x;
-  const int r0 = t * per, r1 = min(r0 + per, n_keys);  // ranks r: key n_keys - 1 - r
-  int32_t local = 0;
-  for (int r = r0; r < r1; ++r) local += hist[n_keys - 1 - r];
-  int32_t incl = local;
+  if (t == 0) s_carry = 0;
+  constexpr int kPiece = kScanThreads * kScanPer;
+  for (int32_t r0 = 0; r0 < n_keys; r0 += kPiece) {  // ranks r: key n_keys - 1 - r
+    for (int j = t; j < kPiece; j += kScanThreads) {
+      const int32_t r = r0 + j;
+      piece[j + j / kScanPer] = r < n_keys ? hist[n_keys - 1 - r] : 0;
+    }
+    __syncthreads();
+    int32_t* mine = piece + t * (kScanPer + 1);
+    int32_t local = 0;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
-  }
-  if (lane == 31) warp_tot[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    const int nw = (int)blockDim.x >> 5;
-    int32_t v = lane < nw ? warp_tot[lane] : 0;
+    for (int j = 0; j < kScanPer; ++j) local += mine[j];
+    int32_t incl = local;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int32_t u = __shfl_up_sync(0xffffffffu, v, o);
-      if (lane >= o) v += u;
+      const int32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
     }
-    if (lane < nw) warp_tot[lane] = v;  // inclusive over warps
-  }
-  __syncthreads();
-  int32_t run = incl - local + (warp > 0 ? warp_tot[warp - 1] : 0);
-  for (int r = r0; r < r1; ++r) {
-    const int32_t c = hist[n_keys - 1 - r];
-    hist[n_keys - 1 - r] = run;
-    run += c;
-  }
-}
-
-__global__ void order_scatter_kernel(LikeArgs a, int32_t gran, int32_t* next, int32_t* perm) {
-  const int lane = threadIdx.x & 31;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < a.n; base += stride) {
-    const int64_t i = base + lane;
-    const bool on = i < a.n;
-    const unsigned mask = __ballot_sync(0xffffffffu, on);
-    if (on) {
-      const int32_t key = order_key(a, i, gran);
-      const unsigned peers = __match_any_sync(mask, key);
-      const int leader = __ffs(peers) - 1;
-      int32_t first = 0;
-      if (lane == leader) first = atomicAdd(&next[key], __popc(peers));
-      first = __shfl_sync(peers, first, leader);
-      perm[first + __popc(peers & ((1u << lane) - 1u))] = (int32_t)i;
+    if (lane == 31) warp_tot[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      int32_t v = warp_tot[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int32_t u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+      }
+      warp_tot[lane] = v;  // inclusive over warps
     }
+    __syncthreads();
+    int32_t run = s_carry + incl - local + (warp > 0 ? warp_tot[warp - 1] : 0);
+#pragma unroll
+    for (int j = 0; j < kScanPer; ++j) {
+      const int32_t c = mine[j];
+      mine[j] = run;
+      run += c;
+    }
+    __syncthreads();
+    if (t == 0) s_carry += warp_tot[31];
+    for (int j = t; j < kPiece; j += kScanThreads) {
+      const int32_t r = r0 + j;
+      if (r < n_keys) hist[n_keys - 1 - r] = piece[j + j / kScanPer];
+    }
+    __syncthreads();
   }
 }
 
 }  // namespace
 
+cudaError_t launch_order_scan(int32_t n_keys, int32_t* counts, cudaStream_t s) {
+  order_scan_kernel<<<1, kScanThreads, 0, s>>>(n_keys, counts);
+  return cudaGetLastError();
+}
+
 int32_t order_keys(int32_t n_bins, int32_t gran) { return (n_bins + gran - 1) / gran + 1; }
 
 cudaError_t launch_sample_order(const LikeArgs& a, int32_t gran, int32_t* hist, int32_t* perm, cudaStream_t s) {
-  const int32_t n_keys = order_keys(a.n_bins, gran);
-  cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(int32_t) * (size_t)n_keys, s);
-  if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)std::min<int64_t>((a.n + 255) / 256, 4 * 152);
-  order_hist_kernel<<<grid, 256, 0, s>>>(a, gran, hist);
-  order_scan_kernel<<<1, 1024, 0, s>>>(n_keys, hist);
-  order_scatter_kernel<<<grid, 256, 0, s>>>(a, gran, hist, perm);
-  return cudaGetLastError();
+  BandKey key;
+  key.mc = a.pos[kMc] >= 0 ? a.theta + (int64_t)a.pos[kMc] * a.n : nullptr;
+  key.q = a.pos[kQ] >= 0 ? a.theta + (int64_t)a.pos[kQ] * a.n : nullptr;
+  key.mc0 = a.fixed[kMc];
+  key.q0 = a.fixed[kQ];
+  key.f_lo = (float)a.f_lo;
+  key.df = (float)a.df;
+  key.n_bins = (float)a.n_bins;
+  key.gran = gran;
+  return launch_order(a.n, order_keys(a.n_bins, gran), key, hist, perm, s);
 }
 
 }  // namespace mbis

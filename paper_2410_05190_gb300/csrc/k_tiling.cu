@@ -9,6 +9,8 @@
 // normalised overlap maximised over a constant phase.
 #include <cuda_fp16.h>
 
+#include "fpkey.cuh"
+#include "order.cuh"
 #include "physics.cuh"
 #include "philox.cuh"
 #include "tc.cuh"
@@ -281,7 +283,9 @@ __device__ __forceinline__ void phase_coeffs_f32(float q, float chi1, float chi2
 
 // Per-sample set-up of the FP16 operand: the live-bin count from the total mass in FP64
 // (FP32 seed, one Newton step: the ISCO cut agrees with FP64 to the bin), the phase
-// coefficients in FP32, the inverse norm from the FP64 prefix table.
+// coefficients in FP32, the inverse norm from the FP64 prefix table.  Bound by the FP64 pipe:
+// reciprocals from an FP32 seed, no library fmod or division, comparisons as integers (2^20
+// points: 157 us before, 104 now).
 struct FastSetup {
   float cf[kNumBasis - 1];
   int32_t kcut;
@@ -290,15 +294,37 @@ struct FastSetup {
 
 __device__ __forceinline__ FastSetup fast_setup(const TilingSpace& sp, const TilingGrid& g, double x, double q) {
   FastSetup o;
-  double mc, qp;
-  map_point(sp, x, q, mc, qp);
-  const double u = (1.0 + qp) * (1.0 + qp) / qp, u3 = u * u * u;
+  // the point's chirp mass and mass ratio (map_point), with one FP64 reciprocal: q and 1/q
+  double mc = x;
+  if (sp.mc_period > 0.0) {
+    const float turns = __fdividef((float)x, (float)sp.mc_period);
+    double r;
+    if (fabsf(turns) < 65536.0f) {  // the quotient's floor to one unit, then exact steps
+      r = fma(-(double)floorf(turns), sp.mc_period, x);
+      if (__double_as_longlong(r) < 0) r += sp.mc_period;
+      if (order_key(r) >= order_key(sp.mc_period)) r -= sp.mc_period;
+    } else {
+      r = fmod(x, sp.mc_period);
+      if (r < 0.0) r += sp.mc_period;
+    }
+    mc = sp.mc_base + r;
+  }
+  const bool swap = order_key(q) < order_key(1.0);
+  const double iq = rcp_refined(q), qp = swap ? iq : q;
+  const double u = q + 2.0 + iq, u3 = u * u * u;   // (1 + q)^2 / q, the same for q and 1/q
   double y = (double)powf((float)u, 0.6f);
   const double y4 = (y * y) * (y * y);
-  y = 0.8 * y + u3 / (5.0 * y4);                   // y^5 = u^3
-  const double m_sec = mc * kTsun * y;
-  o.kcut = live_bins_m(m_sec, g.f_lo, g.df, g.K);
-  const float am = (float)(kPi * m_sec);
+  y -= fma(y4, y, -u3) * (0.2 * (double)rcp_f32((float)y4));  // y^5 = u^3
+  const double a = kPi * kTsun * mc * y;
+  // grid points strictly below the ISCO: an FP32 estimate, then exact FP64 steps
+  const double fi = rcp_refined(a) * (1.0 / 14.696938456699067);
+  const long long fk = order_key(fi);
+  const float kf = ceilf((float)(fi - g.f_lo) * rcp_f32((float)g.df));
+  int32_t k = !(kf > 0.0f) ? 0 : (kf >= (float)g.K ? g.K : (int32_t)kf);
+  while (k > 0 && order_key(fma((double)(k - 1), g.df, g.f_lo)) >= fk) --k;
+  while (k < g.K && order_key(fma((double)k, g.df, g.f_lo)) < fk) ++k;
+  o.kcut = k;
+  const float am = (float)a;
   phase_coeffs_f32((float)qp, (float)sp.chi1, (float)sp.chi2, am, logf(am), cbrtf(am), o.cf);
   o.inv_s = o.kcut > 0 ? rsqrtf((float)(g.w2sum[o.kcut] * g.inv_wref2)) : 0.f;
   return o;
@@ -814,6 +840,18 @@ cudaError_t launch_tiling_setup(const TilingSpace& sp, const TilingGrid& g, int6
   if (n <= 0) return cudaSuccess;
   setup_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(sp, g, n, pts, rec, kc);
   return cudaGetLastError();
+}
+
+namespace {
+struct CountKey {
+  const int32_t* kc;
+  __device__ __forceinline__ int32_t operator()(int64_t i) const { return kc[i]; }
+};
+}  // namespace
+
+cudaError_t launch_tiling_order(int64_t n, const int32_t* kc, int32_t n_keys, int32_t* counts, int32_t* order,
+                                cudaStream_t s) {
+  return launch_order(n, n_keys, CountKey{kc}, counts, order, s);
 }
 
 cudaError_t launch_tiling_assign(const AssignArgs& a, cudaStream_t s) {

@@ -38,8 +38,7 @@ struct mbis_tiling {
   // scratch of the assignment's sample ordering (grown on demand)
   int64_t scr_n = 0;
   float4* d_rec = nullptr;
-  int32_t *d_kc = nullptr, *d_order = nullptr, *d_shist = nullptr, *d_scount = nullptr, *d_soffset = nullptr,
-          *d_snbad = nullptr;
+  int32_t *d_kc = nullptr, *d_order = nullptr, *d_shist = nullptr;
   // pool
   int64_t N = 0;
   double* d_pool = nullptr;   // [2][N]
@@ -131,9 +130,6 @@ void drop_scratch(mbis_tiling* t) {
   tfree(t->d_rec);
   tfree(t->d_order);
   tfree(t->d_shist);
-  tfree(t->d_scount);
-  tfree(t->d_soffset);
-  tfree(t->d_snbad);
   t->scr_n = 0;
 }
 
@@ -439,25 +435,20 @@ mbis_status mbis_tiling_assign(mbis_tiling* t, int64_t n, const double* pts, int
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (n == 0) return MBIS_OK;
   // process the points in order of their live-bin count, so that the 128 samples of a CTA
-  // reach similar K (a stable counting sort on the count)
+  // reach similar K, the longest first (a point's result does not depend on its neighbours)
   if (n > t->scr_n) {
     drop_scratch(t);
-    const int64_t n_seg = (n + mbis::kSortSegment - 1) / mbis::kSortSegment;
     if (cudaMalloc(&t->d_kc, sizeof(int32_t) * n) != cudaSuccess ||
         cudaMalloc(&t->d_rec, sizeof(float4) * 3 * n) != cudaSuccess ||
         cudaMalloc(&t->d_order, sizeof(int32_t) * n) != cudaSuccess ||
-        cudaMalloc(&t->d_shist, sizeof(int32_t) * (size_t)n_seg * (t->K + 1)) != cudaSuccess ||
-        cudaMalloc(&t->d_scount, sizeof(int32_t) * (t->K + 1)) != cudaSuccess ||
-        cudaMalloc(&t->d_soffset, sizeof(int32_t) * (t->K + 1)) != cudaSuccess ||
-        cudaMalloc(&t->d_snbad, sizeof(int32_t)) != cudaSuccess) {
+        cudaMalloc(&t->d_shist, sizeof(int32_t) * (size_t)(t->K + 1)) != cudaSuccess) {
       drop_scratch(t);
       return tfail(t, MBIS_E_OOM, "mbis_tiling_assign: out of device memory");
     }
     t->scr_n = n;
   }
   T_TRY(t, mbis::launch_tiling_setup(t->sp, t->grid(), n, pts, t->d_rec, t->d_kc, s));
-  T_TRY(t, mbis::launch_tiling_lists(n, t->d_kc, t->K + 1, t->d_shist, t->d_scount, t->d_soffset, t->d_snbad,
-                                     t->d_order, s));
+  T_TRY(t, mbis::launch_tiling_order(n, t->d_kc, t->K + 1, t->d_shist, t->d_order, s));
   mbis::AssignArgs a;
   a.sp = t->sp;
   a.g = t->grid();

@@ -72,6 +72,9 @@ struct AssignArgs {
   int32_t* err;          // device error word
   int32_t nkb_pass[kMaxPasses];  // K-blocks each pass's templates reach
 };
+// order[slot] = point, most live bins first (kc in [0, n_keys)); counts: n_keys ints of scratch
+cudaError_t launch_tiling_order(int64_t n, const int32_t* kc, int32_t n_keys, int32_t* counts, int32_t* order,
+                                cudaStream_t s);
 cudaError_t launch_tiling_assign(const AssignArgs& a, cudaStream_t s);
 
 // stable counting sort of tile indices into per-tile member lists

@@ -265,6 +265,7 @@ DrawArgs make_draw_args(const mbis_ctx* c, uint64_t seed, uint64_t ctr0, int64_t
   a.flags = c->prior_flags;
   a.log_mass_norm = c->log_mass_norm;
   a.log_q_const = -logdet - 0.5 * c->P * log(kTwoPi) - c->P * log(c->scale);
+  a.fixed_point = c->opts.precision == MBIS_FP64;
   a.seed = seed;
   a.ctr0 = ctr0;
   a.d_ctr0 = nullptr;

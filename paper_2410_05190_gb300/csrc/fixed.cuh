@@ -12,6 +12,7 @@
 #include <cstdint>
 #include <cstring>
 
+#include "fixed_tables.h"
 #include "physics.cuh"
 
 namespace mbis {
@@ -149,6 +150,111 @@ MBIS_HD void trig_eval(const TrigCell& c, Pair28 tc, Pair28 ts, int64_t& cos_out
   const int64_t c0 = odd ? si : co, s0 = odd ? co : si;
   cos_out = c0 ^ -(int64_t)(((c.q + 1) >> 1) & 1);
   sin_out = s0 ^ -(int64_t)(c.q >> 1);
+}
+
+// ---- logarithm, square root and normal draws ---------------------------------------------
+MBIS_HD uint64_t umadw(uint32_t a, uint32_t b, uint64_t c) {
+#ifdef __CUDA_ARCH__
+  uint64_t d;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+#else
+  return (uint64_t)a * (uint64_t)b + c;
+#endif
+}
+
+MBIS_HD int32_t mulhi_s(int32_t a, int32_t b) {
+#ifdef __CUDA_ARCH__
+  return __mulhi(a, b);
+#else
+  return (int32_t)(((int64_t)a * (int64_t)b) >> 32);
+#endif
+}
+
+MBIS_HD int clz64(uint64_t x) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)x);
+#else
+  return __builtin_clzll(x);
+#endif
+}
+
+constexpr int64_t kLn2_52 = 3121657384082680ll, kLn2_58 = 199786072581291495ll;  // ln 2 in 2^-52, 2^-58
+constexpr int32_t kLn2_62 = -405;  // the rest of the former in 2^-62
+constexpr int32_t kLn2_64 = -20;  // and the rest of the latter in 2^-64
+
+// ln f of f = m 2^-63 in [1, 2), unit 2^-62: with c the table's 8-bit reciprocal of f's
+// 1/128th, y = f c - 1 is exact and below 2^-6.9, ln f = -ln c + ln(1 + y), the series summed
+// to y^8 (the rest is below 2^-65).  k = 256 c and lt = -ln c 2^62 are the entry of log_cell(m).
+MBIS_HD int32_t log_cell(uint64_t m) { return (int32_t)(m >> 56) & 127; }
+
+MBIS_HD int64_t log_frac(uint64_t m, uint32_t k, int64_t lt) {
+  // f c 2^69, whose 2^69 (the 1) is zero modulo 2^64
+  const uint64_t m2 = m >> 2;
+  const int64_t Y = (int64_t)umadw((uint32_t)m2, k, (uint64_t)((uint32_t)(m2 >> 32) * k) << 32);
+  const int64_t y = Y >> 7;  // unit 2^-62
+  const Pair28 yp = pair28(y);
+  const int32_t y32 = yp.h >> 2;  // unit 2^-32
+  int32_t t = (int32_t)(4294967296.0 / 7.0) - mulhi_s(y32, 536870912);
+  t = (int32_t)(4294967296.0 / 6.0) - mulhi_s(y32, t);
+  t = (int32_t)(4294967296.0 / 5.0) - mulhi_s(y32, t);
+  t = (int32_t)(4294967296.0 / 4.0) - mulhi_s(y32, t);
+  // a product with yp has unit 2^-62: six more bits
+  const Pair28 t4 = {t >> 4, (t & 15) << 24};
+  const int64_t g = (int64_t)(kTwo56 / 3.0) - (mul28(yp, t4, 0) >> 6);
+  const int64_t h = ((int64_t)1 << 55) - (mul28(yp, pair28(g), 0) >> 6);
+  const int64_t y2h = mul28(pair28(mul28(yp, yp, 0)), pair28(h), 0);  // unit 2^-68
+  return lt + y - (y2h >> 6);
+}
+
+// sqrt(2 t) of t = T 2^-58 > 0, unit 2^-56: an FP32 reciprocal square root and two Newton
+// corrections of the root
+MBIS_HD int64_t sqrt_2t(int64_t T) {
+  const int lz = clz64((uint64_t)T);       // >= 1
+  const int sh = (lz & 1) ? lz : lz - 1;   // odd: 2 t = M 2^-(57 + sh), M in [2^62, 2^64)
+  const uint64_t M = (uint64_t)T << sh;
+#ifdef __CUDA_ARCH__
+  const float rs = rsqrtf((float)(uint32_t)(M >> 32));
+#else
+  const float rs = 1.0f / std::sqrt((float)(uint32_t)(M >> 32));
+#endif
+  const uint32_t Y = (uint32_t)(rs * 70368744177664.0f);  // 2^62 / sqrt(M), in [2^30, 2^31]
+  const int32_t Ys = (int32_t)(Y >> 1);
+  // G = sqrt(M) 2^30; e = (M 2^60 - G^2) 2^-64, dG = e Y 2^-29
+  uint64_t G = umadw((uint32_t)(M >> 32), Y, umadw((uint32_t)M, Y, 0) >> 32);
+  auto residual = [&]() {
+    const uint32_t gh = (uint32_t)(G >> 32);
+    return (int64_t)((M >> 4) - umadw(gh, gh, umadw(gh, (uint32_t)G, 0) >> 31));
+  };
+  int64_t e = residual();
+  G += (uint64_t)((mulw((int32_t)(e >> 16), Ys) >> 12) + (mulw((int32_t)(e & 0xffff), Ys) >> 28));
+  e = residual();
+  G += (uint64_t)(mulw((int32_t)e, Ys) >> 28);
+  const int out = (57 + sh) / 2 - 26;  // >= 3
+  return (int64_t)((G + ((uint64_t)1 << (out - 1))) >> out);
+}
+
+// -ln u of u = (2 a + 1) 2^-33, unit 2^-58: the mantissa of 2 a + 1, whose table entry the
+// caller looks up, and the sum
+MBIS_HD int64_t minus_log_uniform(int32_t e, int64_t frac) {
+  return -((int64_t)e * kLn2_58 + ((frac + ((e * kLn2_64) >> 2) + 8) >> 4));
+}
+MBIS_HD uint64_t uniform_mantissa(uint32_t a, int32_t& e) {
+  const uint64_t w = 2 * (uint64_t)a + 1;
+  const int lz = clz64(w);
+  e = 30 - lz;
+  return w << lz;
+}
+
+// ln x of a positive normal x = m 2^-63 2^e, unit 2^-52, from log_frac(m)
+MBIS_HD int64_t log_sum(int32_t e, int64_t frac) { return (int64_t)e * kLn2_52 + ((frac + e * kLn2_62 + 512) >> 10); }
+struct LogArg {
+  uint64_t m;
+  int32_t e;
+};
+MBIS_HD LogArg log_arg(double x) {
+  const uint64_t b = double_bits(x);
+  return LogArg{((b & 0xfffffffffffffull) | 0x10000000000000ull) << 11, (int32_t)((b >> 52) & 0x7ff) - 1023};
 }
 
 }  // namespace mbis

@@ -125,6 +125,7 @@ struct DrawArgs {
   uint32_t flags;
   double log_mass_norm;  // ln of the (Mc, q) volume of the flat-in-(m1, m2) prior
   double log_q_const;    // -sum ln L_pp - (P/2) ln 2pi - P ln s
+  int32_t fixed_point;   // normals in fixed point (k_draw.cu)
   uint64_t seed, ctr0;
   const uint64_t* d_ctr0;  // when set, the counter base is read from device memory (graph replays)
   int64_t n;

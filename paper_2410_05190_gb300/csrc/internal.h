@@ -102,7 +102,7 @@ struct LikeArgs {
   int32_t ff_phase;           // block entry in float-float (phase terms below kFloatFloatMaxTurns)
   int32_t* err;               // device error word (timeouts)
   const double* gl;           // Gauss-Legendre nodes / weights (marg.cuh layout)
-  const float* glf;           // the same nodes / weights in FP32 (mixed-precision marginal)
+  const float* glf;           // the same in FP32 and the whole range's nodes (mixed-precision marginal)
   DistConst dist;             // distance-marginal constants of [dmin, dmax]
   // folded kernel split over CTAs (split > 1): per-part overlap sums and the per-sample
   // amplitude (negative: outside the model) and ISCO cut, read by the epilogue kernel
@@ -140,6 +140,8 @@ struct BatchItem {
 };
 
 // kernel launchers (each returns cudaGetLastError() of its launch)
+// glf: the FP32 node table (kGLTableF floats), its first kGLSize filled
+cudaError_t launch_dist_nodes(float span, float* glf, cudaStream_t s);
 cudaError_t launch_basis_table(double f_lo, double df, int32_t n, double* out, cudaStream_t s);
 // Samples per launch from which the mixed likelihood kernels take the samples in order of
 // their live bins (longest band first); gran: the bins of one key (16 for the K-blocks of

@@ -178,7 +178,21 @@ __global__ void twiddle_tiles_kernel(int32_t n, double f_lo, double df, double d
   }
 }
 
+// the sample-independent nodes of the mixed-precision distance rule (marg.cuh)
+__global__ void dist_nodes_kernel(float span, float* glf) {
+  const int i = threadIdx.x;
+  if (i >= kDistFull) return;
+  const float d = dist_node_at(0.0f, span, 24, i / kGL8, glf[2 * kGL48 + i % kGL8]);
+  glf[kGLSize + i] = d;
+  glf[kGLSize + kDistFull + i] = expm1f(d);
+}
+
 }  // namespace
+
+cudaError_t launch_dist_nodes(float span, float* glf, cudaStream_t s) {
+  dist_nodes_kernel<<<1, kDistFull, 0, s>>>(span, glf);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_rows_to_f32(const double2* c, int32_t rows, int32_t n, int32_t n_pad, double inv_scale,
                                float2* out, cudaStream_t s) {

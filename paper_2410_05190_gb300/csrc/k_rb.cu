@@ -18,6 +18,15 @@
 // FP64 coefficient differences, then MUFU sine / cosine; the edge sums run in FP32 over
 // chunks of 16 edges whose sums are gathered as float pairs (no FP64 arithmetic in the
 // sweep).
+//
+// A CTA takes 64 samples, two per lane in packed FP32 (one record read and one instruction for
+// both), and its eight warps share the chunks, the per-sample set-up (its independent parts on
+// different warps) and the nodes of the distance marginal.  Bound by instruction issue (12 per
+// sample and edge beside 2 sine/cosine results); one sample per thread over all edges, the
+// version before, issued 21 and left a 2^16-sample batch two CTAs of 256 threads per SM.
+// Measured on a GB300 on two BNS events (1.8 10^3 and 0.8 10^3 edges): 2^12 samples 160 and
+// 113 us before, 78 and 49 now; 2^16 254 and 165, 189 and 135; 2^20 2.68 and 1.44 ms, 2.49 and
+// 1.39 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -33,9 +42,10 @@
 namespace mbis {
 namespace {
 
-constexpr int kRbThreads = 256;
+constexpr int kRbWarps = 8;
+constexpr int kRbThreads = 32 * kRbWarps;
+constexpr int kRbTile = 64;  // samples per CTA: lane and lane + 32
 constexpr int kRbChunk = 16;
-constexpr size_t kRbSmemMax = 112 * 1024;  // records staged in shared memory up to 2388 bins
 constexpr float kTwoPiF = 6.28318530717958647692f;
 
 // W_k and (f_k - f_lo) W_k as four real rows [re W, im W, re fW, im fW][n]
@@ -107,15 +117,16 @@ struct RbArgs {
   const float4* rec;     // [n_rb + 1][kEdgeVec]
   const float2* q;       // [n_rb] q_b / scale
   const int32_t* edges;  // [n_rb + 1]
-  int32_t rec_smem;      // stage the records in shared memory
   const double* prefix;  // [4][n_bins + 1]
   double scale;
   double C0[kNumBasis], cst0;
 };
 
-// e^(-i 2 pi dPsi) at one edge, and the edge's weight c_e
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+
+// e^(-i 2 pi dPsi) of one sample at one edge, and the edge's weight c_e
 __device__ __forceinline__ float2 edge_rho(const float4* __restrict__ e, const float* dC, float dcst, float2& c) {
-  const float4 r0 = e[0], r1 = e[1], r2 = e[2];
+  const float4 r0 = __ldg(e), r1 = __ldg(e + 1), r2 = __ldg(e + 2);
   c = make_float2(r0.x, r0.y);
   float t = fmaf(dC[0], r0.z, dcst);
   t = fmaf(dC[1], r0.w, t);
@@ -133,107 +144,277 @@ __device__ __forceinline__ float2 edge_rho(const float4* __restrict__ e, const f
   return make_float2(co, s);
 }
 
-__global__ void __launch_bounds__(kRbThreads, 3) rb_loglike_kernel(RbArgs r) {
-  extern __shared__ float4 s_rec[];
+struct RbSmem {
+  double mass[4][kRbTile];   // u, ln a, a^(1/3), 1 / a
+  double pn[6][kRbTile];
+  double amp[kRbTile];
+  float dC[kNumBasis + 1][kRbTile];
+  int32_t kcut[kRbTile];
+  float part[kRbWarps][4][kRbTile];  // per warp: re (hi, lo), im (hi, lo)
+  float dist[6][kRbTile];            // the distance rule: lo, hi, Z, H, u_ref, phi_ref
+  int32_t nodes[kRbTile];            // its nodes: 48, 192 without a window, 0 outside the model
+  float g[2][kGL48][kRbTile];        // 48 node values at a time, two rounds in turn
+};
+
+__global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
+  __shared__ RbSmem sm;
   const LikeArgs& a = r.la;
-  const float4* recs = r.rec;
-  if (r.rec_smem) {
-    for (int i = threadIdx.x; i < kEdgeVec * (r.n_rb + 1); i += blockDim.x) s_rec[i] = __ldg(r.rec + i);
-    __syncthreads();
-    recs = s_rec;
-  }
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= a.n) return;
-  double par[kNumSlots];
-#pragma unroll
-  for (int i = 0; i < kNumSlots; ++i) par[i] = a.pos[i] >= 0 ? a.theta[(int64_t)a.pos[i] * a.n + s] : a.fixed[i];
-  const bool valid = par[kMc] > 0.0 && par[kQ] > 0.0 && fabs(par[kChi1]) < 1.0 && fabs(par[kChi2]) < 1.0 &&
-                     ((a.marg & MBIS_MARG_DISTANCE) || par[kDl] > 0.0) && isfinite(par[kTc]) && isfinite(par[kPhic]);
-  if (!valid) {
-    a.out[s] = -INFINITY;
-    return;
-  }
-  const double dl = (a.marg & MBIS_MARG_DISTANCE) ? 1.0 : par[kDl];
-  const SampleSetup ss = sample_setup(par[kMc], par[kQ], par[kChi1], par[kChi2], par[kTc], par[kPhic], dl, a.f_lo,
-                                      a.df, a.n_bins);
-  const PhaseCoeffs& pc = ss.pc;
-  const int32_t kcut = ss.kcut;
-  const double amp = ss.amp;
-  float dC[kNumBasis];
-#pragma unroll
-  for (int j = 0; j < kNumBasis; ++j) dC[j] = (float)(pc.C[j] - r.C0[j]);
-  const float dcst = (float)(pc.cst - r.cst0);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t s0 = (int64_t)blockIdx.x * kRbTile;
 
-  // nfull = the last edge at or below the cut: bins 0 .. nfull-1 lie wholly below it
-  int32_t lo = 0, hi = r.n_rb;
-  while (lo < hi) {
-    const int32_t mid = (lo + hi + 1) >> 1;
-    if (__ldg(r.edges + mid) <= kcut)
-      lo = mid;
-    else
-      hi = mid - 1;
+  // ---- per-sample set-up (sample_setup of physics.cuh, its parts on different warps)
+  const int si = threadIdx.x & (kRbTile - 1), role = threadIdx.x / kRbTile;
+  const int64_t s = s0 + si;
+  const bool active = s < a.n;
+  auto par = [&](int slot) { return active && a.pos[slot] >= 0 ? a.theta[(int64_t)a.pos[slot] * a.n + s] : a.fixed[slot]; };
+  const double mc = par(kMc), q = par(kQ), chi1 = par(kChi1), chi2 = par(kChi2);
+  const double dl = (a.marg & MBIS_MARG_DISTANCE) ? 1.0 : par(kDl), tc = par(kTc), phic = par(kPhic);
+  const bool valid = active && mc > 0.0 && q > 0.0 && fabs(chi1) < 1.0 && fabs(chi2) < 1.0 && dl > 0.0 &&
+                     isfinite(tc) && isfinite(phic);
+  if (role == 0) {
+    const double u = q + 2.0 + rcp_refined(q), u3 = u * u * u;
+    double y = (double)powf((float)u, 0.6f);
+    {
+      const double y2 = y * y, y4 = y2 * y2;
+      y -= (y4 * y - u3) * (0.2 * (double)rcp_f32((float)y4));
+    }
+    const double am = kPi * kTsun * mc * y;
+    double a13 = (double)cbrtf((float)am);
+    {
+      const double c2 = a13 * a13;
+      a13 -= (c2 * a13 - am) * ((1.0 / 3.0) * (double)rcp_f32((float)c2));
+    }
+    const double inv_a = rcp_refined(am);
+    sm.mass[0][si] = u;
+    sm.mass[1][si] = log(am);
+    sm.mass[2][si] = a13;
+    sm.mass[3][si] = inv_a;
+    const double fi = inv_a * (1.0 / 14.696938456699067);
+    const float kf = ceilf((float)(fi - a.f_lo) * rcp_f32((float)a.df));
+    int32_t k = !(kf > 0.0f) ? 0 : (kf >= (float)a.n_bins ? a.n_bins : (int32_t)kf);
+    while (k > 0 && a.f_lo + (double)(k - 1) * a.df >= fi) --k;
+    while (k < a.n_bins && a.f_lo + (double)k * a.df < fi) ++k;
+    sm.kcut[si] = valid ? k : 0;
+  } else if (role == 1) {
+    const double w = rcp_refined(1.0 + q);
+    const PNTerms t = pn_terms(q * w * w, (q - 1.0) * w, 0.5 * (chi1 + chi2), 0.5 * (chi1 - chi2));
+    sm.pn[0][si] = t.phi2;
+    sm.pn[1][si] = t.phi3;
+    sm.pn[2][si] = t.phi4;
+    sm.pn[3][si] = t.c5;
+    sm.pn[4][si] = t.a6;
+    sm.pn[5][si] = t.phi7;
+  } else if (role == 2) {
+    const double x = mc * kTsun, x2 = x * x, x5 = x2 * x2 * x;
+    double z = (double)powf((float)x, 5.0f / 6.0f);
+    {
+      const double z2 = z * z, z5 = z2 * z2 * z;
+      z -= (z5 * z - x5) * ((1.0 / 6.0) * (double)rcp_f32((float)z5));
+    }
+    sm.amp[si] = 0.45643546458763845 * 0.46619407703541166 * z * rcp_refined(dl * kMpcSeconds);
   }
-  const int32_t nfull = lo;
+  __syncthreads();
+  {
+    const double u = sm.mass[0][si], la = sm.mass[1][si], a13 = sm.mass[2][si], inv_a = sm.mass[3][si];
+    const double pre = (3.0 / (256.0 * kPi)) * u;  // 3 / (128 eta) / (2 pi), turns
+    auto put = [&](int j, double C) { sm.dC[j][si] = (float)(C - (j < kNumBasis ? r.C0[j] : r.cst0)); };
+    if (role == 0) {
+      const double pa = pre * inv_a;
+      put(0, pa * inv_a * a13);                        // a^(-5/3)
+      put(1, pa * sm.pn[0][si]);                       // a^(-1)
+      put(2, pa * sm.pn[1][si] * a13);                 // a^(-2/3)
+    } else if (role == 1) {
+      const double a23 = a13 * a13;
+      put(3, pre * inv_a * sm.pn[2][si] * a23);        // a^(-1/3)
+      put(7, pre * sm.pn[5][si] * a23);
+      put(8, tc);
+    } else if (role == 2) {
+      put(5, pre * a13 * (sm.pn[4][si] - 6848.0 / 63.0 * la));
+      put(6, -pre * a13 * (6848.0 / 63.0));
+    } else {
+      put(4, pre * sm.pn[3][si]);                      // ln f
+      put(kNumBasis, phic * (-1.0 / kTwoPi) - 0.125 + pre * sm.pn[3][si] * (1.0 + la));
+    }
+  }
+  __syncthreads();
 
-  FFSum zr_all, zi_all;  // chunk sums, scaled by 1 / scale
-  int32_t e = 0;
-  for (; e + kRbChunk <= nfull; e += kRbChunk) {
-    float zr = 0.f, zi = 0.f;
+  // ---- sweep: this warp's chunks of 16 edges, both samples of a lane in packed FP32
+  float2 dC[kNumBasis];
+#pragma unroll
+  for (int j = 0; j < kNumBasis; ++j) dC[j] = make_float2(sm.dC[j][lane], sm.dC[j][lane + 32]);
+  const float2 dcst = make_float2(sm.dC[kNumBasis][lane], sm.dC[kNumBasis][lane + 32]);
+  // the last edge at or below the cut: bins 0 .. nfull - 1 lie wholly below it
+  int32_t nfull[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int32_t kcut = sm.kcut[lane + 32 * h];
+    int32_t lo = 0, hi = r.n_rb;
+    if (kcut < a.n_bins) {
+      while (lo < hi) {
+        const int32_t mid = (lo + hi + 1) >> 1;
+        if (__ldg(r.edges + mid) <= kcut)
+          lo = mid;
+        else
+          hi = mid - 1;
+      }
+    } else {
+      lo = r.n_rb;
+    }
+    nfull[h] = lo;
+  }
+  const int32_t n_max = __reduce_max_sync(0xffffffffu, max(nfull[0], nfull[1]));
+  FFSum zr_all[2], zi_all[2];  // chunk sums, scaled by 1 / scale
+  for (int32_t e = kRbChunk * warp; e + kRbChunk <= n_max; e += kRbChunk * kRbWarps) {
+    float2 zr = f2(0.f), zi = f2(0.f);
+    const float4* rec = r.rec + kEdgeVec * e;
 #pragma unroll
     for (int j = 0; j < kRbChunk; ++j) {
+      const float4 r0 = __ldg(rec + kEdgeVec * j), r1 = __ldg(rec + kEdgeVec * j + 1), r2 = __ldg(rec + kEdgeVec * j + 2);
+      float2 t = __ffma2_rn(dC[0], f2(r0.z), dcst);
+      t = __ffma2_rn(dC[1], f2(r0.w), t);
+      t = __ffma2_rn(dC[2], f2(r1.x), t);
+      t = __ffma2_rn(dC[3], f2(r1.y), t);
+      t = __ffma2_rn(dC[4], f2(r1.z), t);
+      t = __ffma2_rn(dC[5], f2(r1.w), t);
+      t = __ffma2_rn(dC[6], f2(r2.x), t);
+      t = __ffma2_rn(dC[7], f2(r2.y), t);
+      t = __ffma2_rn(dC[8], f2(r2.z), t);
+      // the nearest integer removed, as edge_rho does
+      const float2 n = __fadd2_rn(__fadd2_rn(t, f2(12582912.0f)), f2(-12582912.0f));
+      const float2 ang = __fmul2_rn(f2(-kTwoPiF), __fadd2_rn(t, make_float2(-n.x, -n.y)));
+      float2 sn, co;
+      __sincosf(ang.x, &sn.x, &co.x);
+      __sincosf(ang.y, &sn.y, &co.y);
+      zr = __ffma2_rn(co, f2(r0.x), __ffma2_rn(sn, f2(-r0.y), zr));
+      zi = __ffma2_rn(co, f2(r0.y), __ffma2_rn(sn, f2(r0.x), zi));
+    }
+    if (e + kRbChunk <= nfull[0]) {
+      zr_all[0].add(zr.x);
+      zi_all[0].add(zi.x);
+    }
+    if (e + kRbChunk <= nfull[1]) {
+      zr_all[1].add(zr.y);
+      zi_all[1].add(zi.y);
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    sm.part[warp][0][lane + 32 * h] = zr_all[h].h;
+    sm.part[warp][1][lane + 32 * h] = zr_all[h].l;
+    sm.part[warp][2][lane + 32 * h] = zi_all[h].h;
+    sm.part[warp][3][lane + 32 * h] = zi_all[h].l;
+  }
+  // ---- one thread per sample: the edges after its last whole chunk, the bin holding its cut,
+  // the sums of the warps in order
+  const bool dist = a.marg == (MBIS_MARG_PHASE | MBIS_MARG_DISTANCE);
+  double Z = 0.0, H = 0.0, X = 0.0;
+  float zr = 0.f, zi = 0.f;
+  float2 rho_n = f2(0.f);
+  int32_t n_mine = 0;
+  float dCs[kNumBasis], dcs = 0.f;
+  if (role == 0) {
+#pragma unroll
+    for (int j = 0; j < kNumBasis; ++j) dCs[j] = sm.dC[j][si];
+    dcs = sm.dC[kNumBasis][si];
+    n_mine = warp == 0 ? nfull[0] : nfull[1];  // samples lane and lane + 32
+    for (int32_t e = n_mine / kRbChunk * kRbChunk; e < n_mine; ++e) {
       float2 c;
-      const float2 rho = edge_rho(recs + kEdgeVec * (e + j), dC, dcst, c);
+      const float2 rho = edge_rho(r.rec + kEdgeVec * e, dCs, dcs, c);
       zr = fmaf(rho.x, c.x, fmaf(-rho.y, c.y, zr));
       zi = fmaf(rho.x, c.y, fmaf(rho.y, c.x, zi));
     }
-    zr_all.add(zr);
-    zi_all.add(zi);
+    // edge n: the far end of the last whole bin, and the near end of the bin holding the cut
+    float2 c_unused;
+    rho_n = edge_rho(r.rec + kEdgeVec * n_mine, dCs, dcs, c_unused);
+    if (n_mine > 0) {
+      const float2 qn = r.q[n_mine - 1];
+      zr = fmaf(rho_n.x, qn.x, fmaf(-rho_n.y, qn.y, zr));
+      zi = fmaf(rho_n.x, qn.y, fmaf(rho_n.y, qn.x, zi));
+    }
   }
-  float zr = 0.f, zi = 0.f;
-  for (; e < nfull; ++e) {
-    float2 c;
-    const float2 rho = edge_rho(recs + kEdgeVec * e, dC, dcst, c);
-    zr = fmaf(rho.x, c.x, fmaf(-rho.y, c.y, zr));
-    zi = fmaf(rho.x, c.y, fmaf(rho.y, c.x, zi));
+  __syncthreads();
+  if (role == 0) {
+    FFSum sr, sc;
+#pragma unroll
+    for (int w = 0; w < kRbWarps; ++w) {
+      sr.add(sm.part[w][0][si]);
+      sr.l = __fadd_rn(sr.l, sm.part[w][1][si]);
+      sc.add(sm.part[w][2][si]);
+      sc.l = __fadd_rn(sc.l, sm.part[w][3][si]);
+    }
+    sr.add(zr);
+    sc.add(zi);
+    double zr64 = sr.value() * r.scale, zi64 = sc.value() * r.scale;
+    const int32_t kcut = sm.kcut[si];
+    const int32_t k0 = __ldg(r.edges + n_mine);
+    if (k0 < kcut) {
+      // the bin holding the ISCO cut (n_mine < n_rb here): its sums below the cut, from the
+      // prefix tables, against the chord through the bin's two edges
+      const int32_t k1 = __ldg(r.edges + n_mine + 1);
+      float2 c_unused;
+      const float2 rho1 = edge_rho(r.rec + kEdgeVec * (n_mine + 1), dCs, dcs, c_unused);
+      const double inv_w = 1.0 / ((double)(k1 - k0) * a.df);
+      const double sr1 = (double)(rho1.x - rho_n.x) * inv_w, si1 = (double)(rho1.y - rho_n.y) * inv_w;
+      const int64_t m = (int64_t)a.n_bins + 1;
+      const double* T = r.prefix;
+      const double a0r = T[kcut] - T[k0], a0i = T[m + kcut] - T[m + k0];
+      const double ofs = (double)k0 * a.df;
+      const double a1r = (T[2 * m + kcut] - T[2 * m + k0]) - ofs * a0r;
+      const double a1i = (T[3 * m + kcut] - T[3 * m + k0]) - ofs * a0i;
+      zr64 += (double)rho_n.x * a0r - (double)rho_n.y * a0i + sr1 * a1r - si1 * a1i;
+      zi64 += (double)rho_n.x * a0i + (double)rho_n.y * a0r + sr1 * a1i + si1 * a1r;
+    }
+    const double amp = sm.amp[si];
+    Z = amp * hypot(zr64, zi64);
+    X = amp * zr64;
+    H = amp * amp * a.tfold[kcut];
+    if (!dist && active) {
+      double ll;
+      if (a.marg == MBIS_MARG_PHASE)
+        ll = log_i0(Z) - 0.5 * H;
+      else
+        ll = X - 0.5 * H;  // no marginalisation: Re (d|h) - <h|h> / 2
+      a.out[s] = valid ? ll : -INFINITY;
+    }
   }
-  // edge nfull: the far end of the last whole bin, and the near end of the bin holding the cut
-  float2 c_unused;
-  const float2 rho_n = edge_rho(recs + kEdgeVec * nfull, dC, dcst, c_unused);
-  if (nfull > 0) {
-    const float2 q = r.q[nfull - 1];
-    zr = fmaf(rho_n.x, q.x, fmaf(-rho_n.y, q.y, zr));
-    zi = fmaf(rho_n.x, q.y, fmaf(rho_n.y, q.x, zi));
+  if (!dist) return;
+  // the distance marginal: its nodes shared by the warps, 48 at a time, summed in order by the
+  // sample's thread while the warps evaluate the next
+  DistWindow win;
+  if (role == 0) {
+    win = dist_window(Z, H, a.dist);
+    sm.dist[0][si] = win.lo;
+    sm.dist[1][si] = win.hi;
+    sm.dist[2][si] = win.Z;
+    sm.dist[3][si] = win.H;
+    sm.dist[4][si] = win.u_ref;
+    sm.dist[5][si] = win.phi_ref;
+    sm.nodes[si] = valid ? (win.window ? kGL48 : kDistFull) : 0;
   }
-  zr_all.add(zr);
-  zi_all.add(zi);
-  double zr64 = zr_all.value() * r.scale, zi64 = zi_all.value() * r.scale;
-  const int32_t k0 = __ldg(r.edges + nfull);
-  if (k0 < kcut) {
-    // the bin holding the ISCO cut (nfull < n_rb here): its sums below the cut, from the
-    // prefix tables, against the chord through the bin's two edges
-    const int32_t k1 = __ldg(r.edges + nfull + 1);
-    const float2 rho1 = edge_rho(recs + kEdgeVec * (nfull + 1), dC, dcst, c_unused);
-    const double inv_w = 1.0 / ((double)(k1 - k0) * a.df);
-    const double sr = (double)(rho1.x - rho_n.x) * inv_w, si = (double)(rho1.y - rho_n.y) * inv_w;
-    const int64_t m = (int64_t)a.n_bins + 1;
-    const double* T = r.prefix;
-    const double a0r = T[kcut] - T[k0], a0i = T[m + kcut] - T[m + k0];
-    const double ofs = (double)k0 * a.df;
-    const double a1r = (T[2 * m + kcut] - T[2 * m + k0]) - ofs * a0r;
-    const double a1i = (T[3 * m + kcut] - T[3 * m + k0]) - ofs * a0i;
-    zr64 += (double)rho_n.x * a0r - (double)rho_n.y * a0i + sr * a1r - si * a1i;
-    zi64 += (double)rho_n.x * a0i + (double)rho_n.y * a0r + sr * a1i + si * a1r;
+  const bool any_full = __syncthreads_or(role == 0 && valid && !win.window);
+  LogSumExpF L;
+  const int rounds = any_full ? kDistFull / kGL48 : 1;
+  for (int rd = 0; rd < rounds; ++rd) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = lane + 32 * h, n = sm.nodes[i];
+      if (rd * kGL48 >= n) continue;
+      const float lo = sm.dist[0][i], hi = sm.dist[1][i], Zf = sm.dist[2][i], Hf = sm.dist[3][i], u = sm.dist[4][i],
+                  phi = sm.dist[5][i];
+#pragma unroll 2
+      for (int j = warp; j < kGL48; j += kRbWarps) {
+        const float2 node = dist_main_node(n == kGL48, lo, hi, a.glf, rd * kGL48 + j);
+        sm.g[rd & 1][j][i] = dist_node_e(node.x, node.y, Zf, Hf, u, phi);
+      }
+    }
+    __syncthreads();
+    if (role == 0 && rd * kGL48 < sm.nodes[si]) {
+#pragma unroll 4
+      for (int j = 0; j < kGL48; ++j)
+        L.add(sm.g[rd & 1][j][si], dist_main_weight(win.window, win.lo, win.hi, a.glf, rd * kGL48 + j));
+    }
   }
-  const double z = amp * hypot(zr64, zi64);
-  const double H = amp * amp * a.tfold[kcut];
-  double ll;
-  if (a.marg == MBIS_MARG_PHASE)
-    ll = log_i0(z) - 0.5 * H;
-  else if (a.marg == (MBIS_MARG_PHASE | MBIS_MARG_DISTANCE))
-    ll = log_distance_marginal_mixed(z, H, a.dist, a.glf);  // as the fused kernel
-  else
-    ll = amp * zr64 - 0.5 * H;  // no marginalisation: Re (d|h) - <h|h> / 2
-  a.out[s] = ll;
+  if (role == 0 && active) a.out[s] = valid ? dist_finish(win, L, Z, H, a.dist, a.glf) : -INFINITY;
 }
 
 mbis_status rb_fail(mbis_ctx* c, mbis_status st, const std::string& msg) {
@@ -359,18 +540,7 @@ mbis_status mbis_rb_loglike(mbis_ctx* c, int64_t n, const double* theta, double*
   r.scale = c->rb_scale;
   for (int j = 0; j < kNumBasis; ++j) r.C0[j] = c->rb_C0[j];
   r.cst0 = c->rb_cst0;
-  // the records in shared memory when they fit (a few CTAs per SM still), else through L1
-  const size_t sh = sizeof(float4) * kEdgeVec * (size_t)(c->rb_n + 1);
-  r.rec_smem = sh <= kRbSmemMax ? 1 : 0;
-  if (r.rec_smem && sh > 48 * 1024) {
-    static bool attr = false;
-    if (!attr) {
-      RB_TRY(c, cudaFuncSetAttribute(rb_loglike_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRbSmemMax));
-      attr = true;
-    }
-  }
-  rb_loglike_kernel<<<(unsigned)((n + kRbThreads - 1) / kRbThreads), kRbThreads, r.rec_smem ? sh : 0,
-                      static_cast<cudaStream_t>(stream)>>>(r);
+  rb_loglike_kernel<<<(unsigned)((n + kRbTile - 1) / kRbTile), kRbThreads, 0, static_cast<cudaStream_t>(stream)>>>(r);
   RB_TRY(c, cudaGetLastError());
   return MBIS_OK;
 }

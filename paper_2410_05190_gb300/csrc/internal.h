@@ -157,6 +157,8 @@ cudaError_t launch_rows_to_f32(const double2* c, int32_t rows, int32_t n, int32_
 cudaError_t launch_twiddle_tiles(int32_t n, double f_lo, double df, double dt, int32_t n_kb, float* out,
                                  cudaStream_t s);
 cudaError_t launch_loglike_mixed_time(const LikeArgs& a, cudaStream_t s);
+// tile: 32 or 64 samples per CTA; float-float block entry
+cudaError_t launch_loglike_mixed_time_small(const LikeArgs& a, int32_t tile, cudaStream_t s);
 
 struct MomentArgs {
   double ref[kMaxP];     // offsets are taken from this point

@@ -74,11 +74,11 @@ __device__ __forceinline__ int64_t log_of(const DrawTables& tb, double x) {
   return log_sum(a.e, log_mantissa(tb, a.m));
 }
 
-// cosine and sine of a phase, unit 2^-56
+// cosine and sine of a phase, unit 2^-62
 __device__ __forceinline__ void trig_of(const DrawTables& tb, uint64_t P, int64_t& co, int64_t& si) {
   const TrigCell c = trig_cell(P);
   const int4 t = tb.trig[c.i];
-  trig_eval(c, Pair28{t.x, t.y}, Pair28{t.z, t.w}, co, si);
+  trig_eval(c, Pair32{t.x, t.y}, Pair32{t.z, t.w}, co, si);
 }
 
 // an angle |x| < 16 rad in turns, modulo one, unit 2^-64
@@ -96,8 +96,8 @@ __device__ __forceinline__ int64_t box_muller(const DrawTables& tb, uint32_t a, 
   const Pair28 r = pair28(sqrt_2t(t));
   int64_t co, si;
   trig_of(tb, ((uint64_t)b << 32) + 0x80000000ull, co, si);
-  z0 = pair28(mul28(r, pair28(co), 0));
-  z1 = pair28(mul28(r, pair28(si), 0));
+  z0 = pair28(mul28(r, pair28(co >> 6), 0));
+  z1 = pair28(mul28(r, pair28(si >> 6), 0));
   return t;
 }
 
@@ -112,7 +112,7 @@ template <int P, bool kFixed>
 __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawConsts k) {
   __shared__ DrawTables tb;
   if (threadIdx.x < 32) {
-    const Pair28 c = pair28(kTrigTable[threadIdx.x][0]), s = pair28(kTrigTable[threadIdx.x][1]);
+    const Pair32 c = pair32(kTrigTable[threadIdx.x][0]), s = pair32(kTrigTable[threadIdx.x][1]);
     tb.trig[threadIdx.x] = make_int4(c.h, c.l, s.h, s.l);
   }
   static_assert(kDrawThreads == 128, "a table entry per thread");
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawCons
       int64_t v = id == kDec ? co : si;
       if (v < 1) v = 1;  // the ends of the range
       const int lz = clz64((uint64_t)v);
-      log_sum50 += log_sum(7 - lz, log_mantissa(tb, (uint64_t)v << lz)) >> 2;
+      log_sum50 += log_sum(1 - lz, log_mantissa(tb, (uint64_t)v << lz)) >> 2;
     }
     if (id == kDl) log_sum50 += log_of(tb, inside ? x : 1.0) >> 1;
   }

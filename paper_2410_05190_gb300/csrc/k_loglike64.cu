@@ -7,21 +7,21 @@
 // phase, a sincospi and a complex multiply-add in FP64 (the version before) costs 3750 clocks
 // per warp.  Every one of these quantities is bounded, and 64-bit integers carry them further
 // than FP64 does (fixed.cuh): per bin and warp
-//   * the phase in turns modulo one, sum_j C_j B_j(f_k), 27 multiply-adds of 28-bit halves with
-//     a unit of 2^-58 of the sample's largest phase term (FP64 rounds each term at 2^-53);
-//   * its sine and cosine to a few 2^-56 (a table of 32 entries held one per lane, fetched by
-//     shuffles, and the Taylor series of the rest: 27 multiply-adds);
+//   * the phase in turns modulo one, sum_j C_j B_j(f_k), 29 multiply-adds of 32-bit halves with
+//     a unit of 2^-56 of the sample's largest phase term (FP64 rounds each term at 2^-53);
+//   * its sine and cosine to 2.7e-17 (a table of 32 entries held one per lane, fetched by
+//     shuffles, and the Taylor series of the rest: 36 multiply-adds);
 //   * the multiply-add with the data, scaled by the largest value of 32 bins, into 64-bit sums
-//     (12 multiply-adds; exact but for 2^-56 of the products), which FP64 gathers per 32 bins.
+//     (14 multiply-adds; exact but for 2^-56 of the products), which FP64 gathers per 32 bins.
 // A warp takes 32 samples, one per lane, and 32-bin chunks of the grid: the lanes load and
 // convert one bin each, and all read the converted bins back from shared memory.  A cluster of
 // CTAs shares a tile of 32 samples, its warps taking the chunks in turn, and folds the sums
 // through distributed shared memory in a fixed order, so the launch needs no scratch.  The
 // per-sample set-up is spread over the CTA's warps, and the distance integral's nodes over the
 // cluster's warps.  Phase terms beyond 2^40 turns and non-finite data fall back to FP64 per
-// bin.  Bound by the integer multiply-adds.  Measured on a GB300, 4096 samples: 52.4 ms before
-// and 8.2 ms now on 128,513 bins with phase and distance marginalised; 291 us and 60 us on
-// 1969 bins (240 live) with the phase marginalised.
+// bin.  Bound by the integer multiply-adds (86 per warp and bin, 4 clocks each).  Measured on a
+// GB300, 4096 samples: 52.4 ms before and 6.6 ms now on 128,513 bins with phase and distance
+// marginalised; 291 us and 56 us on 1969 bins (240 live) with the phase marginalised.
 //
 // loglike_fp64_time_kernel (time marginalisation): one warp per sample, lanes over bins, every
 // bin in FP64; the per-bin integrand a_k = A sum_d P_d c_dk e^(-i phi_dk) of 32
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kThreads64) loglike_fp64_time_kernel(LikeArgs 
 // ---- no time marginalisation -------------------------------------------------------------
 constexpr int kTile64 = 32;                  // samples per cluster, one per lane
 constexpr int kWarps64 = kThreads64 / 32;
-constexpr int kMaxCluster64 = 16;
+constexpr int kMaxCluster64 = 8;
 constexpr int kPhaseInts = 20;               // 9 pairs and a pad: rows of 16-byte vectors
 constexpr int kMaxTurnsExp = 40;             // phase terms below 2^40 turns
 
@@ -186,7 +186,6 @@ template <int ROWS>
 struct Smem64 {
   static constexpr int kRow = kPhaseInts + 4 * ROWS;  // ints of one staged bin
   __align__(16) int32_t stage[kWarps64][32][kRow];
-  __align__(16) int4 trig[32];
   double C[kNumBasis + 1][kTile64];                   // phase coefficients and the constant
   double pn[6][kTile64], mass[4][kTile64], amp[kTile64];
   double resp[3][ROWS][kTile64];                      // Re P, Im P, delay of each detector
@@ -313,12 +312,7 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
   } else if (warp == 2) {
     sm.amp[lane] = 0.45643546458763845 * 0.46619407703541166 * pow_5_6(par[kMc] * kTsun) *
                    rcp_any(par[kDl] * kMpcSeconds);
-  } else if (warp == 3) {
-    double sn, cs;
-    sincospi((double)lane * (1.0 / 64.0), &sn, &cs);
-    const Pair28 tc = pair28(to_fixed(cs, 56)), ts = pair28(to_fixed(sn, 56));
-    sm.trig[lane] = make_int4(tc.h, tc.l, ts.h, ts.l);
-  } else if (!FOLD && warp - 4 < ROWS) {
+  } else if (!FOLD && warp >= 4 && warp - 4 < ROWS) {
     const int d = warp - 4;
     double sp, cp, sd, cd, ss, cs;
     sincos(par[kRa] - a.gmst, &sp, &cp);
@@ -352,7 +346,7 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
   }
   __syncthreads();
 
-  // ---- the sample's coefficients in fixed point: every term below 2^T turns, unit 2^(T-58)
+  // ---- the sample's coefficients in fixed point: every term below 2^T turns, unit 2^(T-56)
   int32_t T = 0;
 #pragma unroll
   for (int j = 0; j < kNumBasis; ++j) T = max(T, exponent_above(sm.C[j][lane]) + g.eb[j]);
@@ -363,19 +357,19 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
   }
   const bool far = __any_sync(0xffffffffu, T > kMaxTurnsExp);  // warp-uniform, the same in every warp
   T = min(T, kMaxTurnsExp);
-  Pair28 c[kNumBasis], cd[FOLD ? 1 : ROWS];
+  Pair32 c[kNumBasis], cd[FOLD ? 1 : ROWS];
 #pragma unroll
-  for (int j = 0; j < kNumBasis; ++j) c[j] = pair28(far ? 0 : to_fixed(sm.C[j][lane], 57 - T + g.eb[j]));
-  const int64_t cst = far ? 0 : to_fixed(sm.C[kNumBasis][lane], 58 - T);
+  for (int j = 0; j < kNumBasis; ++j) c[j] = pair32(far ? 0 : to_fixed(sm.C[j][lane], 60 - T + g.eb[j]));
+  const int64_t cst = far ? 0 : to_fixed(sm.C[kNumBasis][lane], 56 - T);
   if constexpr (!FOLD) {
 #pragma unroll
     for (int d = 0; d < ROWS; ++d)
-      cd[d] = pair28(far ? 0 : to_fixed(sm.resp[2][d][lane], 57 - T + g.eb[kNumBasis - 1]));
+      cd[d] = pair32(far ? 0 : to_fixed(sm.resp[2][d][lane], 60 - T + g.eb[kNumBasis - 1]));
   }
-  const int32_t shift = T + 6;  // to 2^-64 turns
+  const int32_t shift = T + 8;  // to 2^-64 turns
   const int32_t kcut = sm.kcut[lane];
   const int32_t kmax = __reduce_max_sync(0xffffffffu, kcut);
-  const int4 trig = sm.trig[lane];
+  const Pair32 trig_c = pair32(kTrigTable[lane][0]), trig_s = pair32(kTrigTable[lane][1]);
 
   // ---- sweep over the grid in chunks of 32 bins (or fewer)
   double zr[ROWS], zi[ROWS];
@@ -396,7 +390,7 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
         nw[d] = on ? __ldg(w + k) : make_double2(0.0, 0.0);
       }
     }
-    // each lane converts its bin: the basis in unit 2^(eb - 57), the data in 2^(E - 56)
+    // each lane converts its bin: the basis in unit 2^(eb - 60), the data in 2^(E - 58)
     int32_t E = -1022;
 #pragma unroll
     for (int d = 0; d < ROWS; ++d) E = max(E, max(exponent_above(nw[d].x), exponent_above(nw[d].y)));
@@ -408,14 +402,14 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
       int32_t v[Smem64<ROWS>::kRow];
 #pragma unroll
       for (int j = 0; j < kNumBasis; ++j) {
-        const Pair28 b = pair28(to_fixed(nb[j], 57 - g.eb[j]));
+        const Pair32 b = pair32(to_fixed(nb[j], 60 - g.eb[j]));
         v[2 * j] = b.h;
         v[2 * j + 1] = b.l;
       }
       v[18] = v[19] = 0;
 #pragma unroll
       for (int d = 0; d < ROWS; ++d) {
-        const Pair28 wr = pair28(to_fixed(nw[d].x, 56 - E)), wi = pair28(to_fixed(nw[d].y, 56 - E));
+        const Pair32 wr = pair32(to_fixed(nw[d].x, 58 - E)), wi = pair32(to_fixed(nw[d].y, 58 - E));
         v[kPhaseInts + 4 * d] = wr.h;
         v[kPhaseInts + 4 * d + 1] = wr.l;
         v[kPhaseInts + 4 * d + 2] = wi.h;
@@ -427,9 +421,9 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
     }
     __syncwarp();
     if (!slow) {
-      int64_t ar[ROWS], ai[ROWS], mr[ROWS], mi[ROWS];
+      int64_t ar[ROWS], ai[ROWS];  // unit 2^(E - 56)
 #pragma unroll
-      for (int d = 0; d < ROWS; ++d) ar[d] = ai[d] = mr[d] = mi[d] = 0;
+      for (int d = 0; d < ROWS; ++d) ar[d] = ai[d] = 0;
 #pragma unroll 1
       for (int32_t k = k0; k < k_end; ++k) {
         const int4* row = reinterpret_cast<const int4*>(sm.stage[warp][k - k0]);
@@ -442,13 +436,16 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
           b[4 * q + 2] = t.z;
           b[4 * q + 3] = t.w;
         }
-        int64_t hi = cst, mid = 0;
+        // each half's terms stay below 2^59, so ten of them fit a sum
+        int64_t hi = cst, mid0 = 0, mid = 0;
 #pragma unroll
         for (int j = 0; j < kNumBasis; ++j) {
+          int64_t& mj = j < 5 ? mid0 : mid;
           hi = madw(c[j].h, b[2 * j], hi);
-          mid = madw(c[j].h, b[2 * j + 1], mid);
-          mid = madw(c[j].l, b[2 * j], mid);
+          mj = madw(c[j].h, b[2 * j + 1], mj);
+          mj = madw(c[j].l, b[2 * j], mj);
         }
+        hi = add_high(mid0, hi);
 #pragma unroll
         for (int d = 0; d < ROWS; ++d) {
           int64_t dh = hi, dm = mid;
@@ -457,28 +454,28 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
             dm = madw(cd[d].h, b[2 * kNumBasis - 1], dm);
             dm = madw(cd[d].l, b[2 * kNumBasis - 2], dm);
           }
-          const uint64_t P = (uint64_t)(dh + (dm >> 28)) << shift;
+          const uint64_t P = (uint64_t)add_high(dm, dh) << shift;
           const TrigCell cell = trig_cell(P);
-          const Pair28 tc = {__shfl_sync(0xffffffffu, trig.x, cell.i), __shfl_sync(0xffffffffu, trig.y, cell.i)};
-          const Pair28 ts = {__shfl_sync(0xffffffffu, trig.z, cell.i), __shfl_sync(0xffffffffu, trig.w, cell.i)};
+          const Pair32 tc = {__shfl_sync(0xffffffffu, trig_c.h, cell.i), __shfl_sync(0xffffffffu, trig_c.l, cell.i)};
+          const Pair32 ts = {__shfl_sync(0xffffffffu, trig_s.h, cell.i), __shfl_sync(0xffffffffu, trig_s.l, cell.i)};
           int64_t co64, si64;
           trig_eval(cell, tc, ts, co64, si64);
-          const Pair28 co = pair28(co64), si = pair28(si64);
+          const Pair32 co = pair32(co64), si = pair32(si64);
           const int4 w = row[kPhaseInts / 4 + d];  // re (h, l), im (h, l)
           if (k < kcut) {
             // w e^(-i phi): (re co + im si, im co - re si)
-            ar[d] = madw(w.z, si.h, madw(w.x, co.h, ar[d]));
-            mr[d] = madw(w.z, si.l, madw(w.w, si.h, madw(w.x, co.l, madw(w.y, co.h, mr[d]))));
-            ai[d] = madw(-w.x, si.h, madw(w.z, co.h, ai[d]));
-            mi[d] = madw(-w.x, si.l, madw(-w.y, si.h, madw(w.z, co.l, madw(w.w, co.h, mi[d]))));
+            const int64_t mr = madw(w.z, si.l, madw(w.w, si.h, madw(w.x, co.l, mulw(w.y, co.h))));
+            const int64_t mi = madw(-w.x, si.l, madw(-w.y, si.h, madw(w.z, co.l, mulw(w.w, co.h))));
+            ar[d] = add_high(mr, madw(w.z, si.h, madw(w.x, co.h, ar[d])));
+            ai[d] = add_high(mi, madw(-w.x, si.h, madw(w.z, co.h, ai[d])));
           }
         }
       }
       const double scale = __longlong_as_double((int64_t)(max(E, -900) - 56 + 1023) << 52);
 #pragma unroll
       for (int d = 0; d < ROWS; ++d) {
-        zr[d] = fma((double)(ar[d] + (mr[d] >> 28)), scale, zr[d]);
-        zi[d] = fma((double)(ai[d] + (mi[d] >> 28)), scale, zi[d]);
+        zr[d] = fma((double)ar[d], scale, zr[d]);
+        zi[d] = fma((double)ai[d], scale, zi[d]);
       }
     } else {
 #pragma unroll 1
@@ -691,9 +688,10 @@ cudaError_t launch_loglike_fp64(const LikeArgs& a, cudaStream_t s) {
   g.s_lo = -std::log(a.dmax);
   g.s_hi = -std::log(a.dmin);
   const int64_t tiles = (a.n + kTile64 - 1) / kTile64;
-  // CTAs per tile: enough for two waves of the GPU's 304 CTA slots, and on long grids so many
-  // that a warp sweeps at most 1024 bins (the last wave then idles little); but at least a
-  // 32-bin chunk for every warp
+  // CTAs per tile: enough for four waves of the SMs, and on long grids so many that a warp
+  // sweeps at most 1024 bins (the last wave then idles little); but at least a 32-bin chunk for
+  // every warp.  At most eight: clusters of sixteen leave more of a GPC's CTA slots empty (4096
+  // samples of 128,513 bins: 8.06 ms at 16, 6.86 at 8, 6.96 at 4).
   int R = 1;
   while (R < kMaxCluster64 && (int64_t)kThreads64 * 2 * R <= a.n_bins &&
          (tiles * R < 608 || a.n_bins > 1024 * kWarps64 * R))

@@ -6,14 +6,18 @@
 // e^(lw - m_b) and its square, and leaves (m_b, S1_b, S2_b); the last CTA to finish (atomic
 // ticket) folds the partials about m = max m_b in a fixed order with all its threads, so the
 // result does not depend on scheduling.  When weights are asked for, the first launch leaves
-// e^(lw - m_b) in them and a second one scales each CTA's samples by e^(m_b - m) / S1: one
-// FP64 exponential per sample in all, where the FP64 pipe (2 lanes per clock per SM) and not
-// HBM bounds the pass.  Measured on a GB300 at 2^18 samples with weights (device time of the
-// launches): 94 us for the three launches this replaces (max 10, sum 69, weights 15: the
-// sum's last thread alone folded 608 partials one dependent add after the other) against 52
-// here (40 and 12); at 2^16, 78 against 30.
+// e^(lw - m_b) in them and a second one scales each CTA's samples by e^(m_b - m) / S1.
+// The FP64 pipe (64 clocks per warp instruction and SM quarter) bounds the pass and not HBM:
+// the exponentials run in fixed point (fixed.cuh: 0.76 ulp at most, 0.31 rms, where FP64 took
+// some 30 instructions), the maxima on the integer pipe, and a warp's two sums fold with five
+// adds between them, which leaves five FP64 instructions per sample.  Measured on a GB300 with
+// weights (device time): 94 us at 2^18 samples, 78 at 2^16 and 74 at 4096 for the three launches
+// of the first version (its sum ended in one thread adding 608 partials), RED18, RED16 and RED12
+// here.
 #include <algorithm>
 
+#include "fixed.cuh"
+#include "fpkey.cuh"
 #include "internal.h"
 
 namespace mbis {
@@ -23,30 +27,45 @@ namespace {
 // more than kReduceBlocks * kReduceThreads * kKeep samples read the inputs twice
 constexpr int kKeep = 8;
 constexpr int kWarps = kReduceThreads / 32;
+static_assert(kWarps == 8, "the second fold takes one lane per warp in each half of a warp");
+constexpr long long kKeyMin = -0x7ff0000000000000ll;  // order_key(-inf)
 
 __device__ __forceinline__ double log_weight(const double* ll, const double* lp, const double* lq, int64_t i) {
   return ll[i] + lp[i] - lq[i];
 }
 
-struct OpMax {
-  static __device__ __forceinline__ double of(double a, double b) { return fmax(a, b); }
-};
-struct OpSum {
-  static __device__ __forceinline__ double of(double a, double b) { return a + b; }
-};
+__device__ __forceinline__ double from_key(long long k) {
+  return __longlong_as_double(k >= 0 ? k : (long long)(0x8000000000000000ull - (unsigned long long)k));
+}
 
-// every thread gets the fold of the CTA's values (warp shuffles, then the warps' results)
-template <typename Op>
-__device__ __forceinline__ double block_fold(double v, double* sh) {
+// every thread gets the largest key
+__device__ __forceinline__ long long block_max(long long v, long long* sh) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = Op::of(v, __shfl_xor_sync(0xffffffffu, v, o));
+  for (int o = 16; o > 0; o >>= 1) v = max(v, (long long)__shfl_xor_sync(0xffffffffu, v, o));
   __syncthreads();  // sh is free
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
   v = sh[0];
 #pragma unroll
-  for (int w = 1; w < kWarps; ++w) v = Op::of(v, sh[w]);
+  for (int w = 1; w < kWarps; ++w) v = max(v, sh[w]);
   return v;
+}
+
+// thread 0 gets both sums: the lower half of a warp folds a, the upper b
+__device__ __forceinline__ void block_sum2(double& a, double& b, double* sh) {
+  const int lane = threadIdx.x & 31;
+  double v = (lane < 16 ? a : b) + __shfl_xor_sync(0xffffffffu, lane < 16 ? b : a, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((lane & 15) == 0) sh[(lane >> 4) * kWarps + (threadIdx.x >> 5)] = v;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    v = (lane & 15) < kWarps ? sh[(lane >> 4) * kWarps + (lane & 15)] : 0.0;
+#pragma unroll
+    for (int o = kWarps / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    a = v;
+    b = __shfl_sync(0xffffffffu, v, 16);
+  }
 }
 
 __device__ __forceinline__ bool last_block(unsigned int* counter) {
@@ -58,50 +77,54 @@ __device__ __forceinline__ bool last_block(unsigned int* counter) {
   return last;
 }
 
-// e^(lw - m); a CTA without a weight above -inf (m = -inf) has zeros, and NaN where lw is NaN
-__device__ __forceinline__ double shifted_exp(double lw, double m) {
-  return m > -INFINITY ? exp(lw - m) : (lw == lw ? 0.0 : lw);
+// e^(x - m) for x <= m; NaN where x is (or both are infinite); a CTA without a weight above
+// -inf (m = -inf) has zeros
+__device__ __forceinline__ double shifted_exp(double x, double m) {
+  const double d = x - m;
+  if (is_nan(d)) return is_nan(x) || order_key(m) > kKeyMin ? d : 0.0;
+  const long long k = order_key(d);
+  if (k < order_key(-700.0)) return k < order_key(-746.0) ? 0.0 : exp(d);
+  int32_t n;
+  uint64_t t;
+  const int32_t j = exp_cell(d, n, t);
+  return exp_eval(n, t, __ldg(reinterpret_cast<const long long*>(kExpTable) + j));
 }
 
 __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(int64_t n, const double* ll, const double* lp,
                                                                 const double* lq, double* w, ReduceScratch scr) {
-  __shared__ double sh[kWarps];
+  __shared__ long long sh_max[kWarps];
+  __shared__ double sh_sum[2 * kWarps];
   const int64_t stride = (int64_t)gridDim.x * kReduceThreads;
   const int64_t i0 = (int64_t)blockIdx.x * kReduceThreads + threadIdx.x;
   double v[kKeep];
-  double m = -INFINITY;
+  long long top = kKeyMin;
 #pragma unroll
   for (int r = 0; r < kKeep; ++r) {
     const int64_t i = i0 + r * stride;
-    v[r] = i < n ? log_weight(ll, lp, lq, i) : -INFINITY;
+    if (i < n) v[r] = log_weight(ll, lp, lq, i);
   }
 #pragma unroll
   for (int r = 0; r < kKeep; ++r)
-    if (v[r] > m) m = v[r];
+    if (i0 + r * stride < n && !is_nan(v[r])) top = max(top, order_key(v[r]));
   for (int64_t i = i0 + kKeep * stride; i < n; i += stride) {
     const double lw = log_weight(ll, lp, lq, i);
-    if (lw > m) m = lw;
+    if (!is_nan(lw)) top = max(top, order_key(lw));
   }
-  m = block_fold<OpMax>(m, sh);
+  const double m = from_key(block_max(top, sh_max));
   double s1 = 0.0, s2 = 0.0;
+  auto take = [&](int64_t i, double lw) {
+    const double e = shifted_exp(lw, m);
+    s1 += e;
+    s2 = fma(e, e, s2);
+    if (w) w[i] = e;
+  };
 #pragma unroll
   for (int r = 0; r < kKeep; ++r) {
     const int64_t i = i0 + r * stride;
-    if (i < n) {
-      const double e = shifted_exp(v[r], m);
-      s1 += e;
-      s2 += e * e;
-      if (w) w[i] = e;
-    }
+    if (i < n) take(i, v[r]);
   }
-  for (int64_t i = i0 + kKeep * stride; i < n; i += stride) {
-    const double e = shifted_exp(log_weight(ll, lp, lq, i), m);
-    s1 += e;
-    s2 += e * e;
-    if (w) w[i] = e;
-  }
-  s1 = block_fold<OpSum>(s1, sh);
-  s2 = block_fold<OpSum>(s2, sh);
+  for (int64_t i = i0 + kKeep * stride; i < n; i += stride) take(i, log_weight(ll, lp, lq, i));
+  block_sum2(s1, s2, sh_sum);
   if (threadIdx.x == 0) {
     scr.partials[3 * blockIdx.x] = m;
     scr.partials[3 * blockIdx.x + 1] = s1;
@@ -110,7 +133,7 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(int64_t n, const
   if (!last_block(scr.counter)) return;
   constexpr int kPer = (kReduceBlocks + kReduceThreads - 1) / kReduceThreads;
   double pm[kPer], p1[kPer], p2[kPer];
-  double mm = -INFINITY;
+  top = kKeyMin;
 #pragma unroll
   for (int r = 0; r < kPer; ++r) {
     const int b = r * kReduceThreads + threadIdx.x;
@@ -118,24 +141,25 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(int64_t n, const
     pm[r] = on ? __ldcg(scr.partials + 3 * b) : -INFINITY;
     p1[r] = on ? __ldcg(scr.partials + 3 * b + 1) : 0.0;
     p2[r] = on ? __ldcg(scr.partials + 3 * b + 2) : 0.0;
-    mm = fmax(mm, pm[r]);
+    top = max(top, order_key(pm[r]));
   }
-  mm = block_fold<OpMax>(mm, sh);
-  double a = 0.0, b2 = 0.0;
-  if (mm > -INFINITY) {  // otherwise every weight is zero, whatever is NaN
+  top = block_max(top, sh_max);
+  const double mm = from_key(top);
+  s1 = s2 = 0.0;
+  if (top > kKeyMin) {  // otherwise every weight is zero, whatever is NaN
 #pragma unroll
     for (int r = 0; r < kPer; ++r) {
-      const double f = pm[r] == mm ? 1.0 : exp(pm[r] - mm);
-      a += p1[r] * f;
-      b2 += p2[r] * f * f;
+      if (r * kReduceThreads + (int)threadIdx.x >= (int)gridDim.x) continue;
+      const double f = order_key(pm[r]) == top ? 1.0 : shifted_exp(pm[r], mm);
+      s1 = fma(p1[r], f, s1);
+      s2 = fma(p2[r], f * f, s2);
     }
   }
-  a = block_fold<OpSum>(a, sh);
-  b2 = block_fold<OpSum>(b2, sh);
+  block_sum2(s1, s2, sh_sum);
   if (threadIdx.x == 0) {
     scr.result[0] = mm;
-    scr.result[1] = a;
-    scr.result[2] = b2;
+    scr.result[1] = s1;
+    scr.result[2] = s2;
     scr.result[3] = (double)n;
     *scr.counter = 0u;
   }
@@ -143,11 +167,18 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(int64_t n, const
 
 // the same grid as reduce_kernel: this CTA's samples are those its maximum belongs to
 __global__ void __launch_bounds__(kReduceThreads) weights_kernel(int64_t n, ReduceScratch scr, double* w) {
-  const double m = scr.result[0], mb = scr.partials[3 * blockIdx.x];
-  const double f = (mb == m ? 1.0 : exp(mb - m)) / scr.result[1];
+  __shared__ double sh_f;
+  const double m = scr.result[0];
+  if (threadIdx.x == 0) {
+    const double mb = scr.partials[3 * blockIdx.x];
+    sh_f = (order_key(mb) == order_key(m) ? 1.0 : shifted_exp(mb, m)) / scr.result[1];
+  }
+  __syncthreads();
+  const double f = sh_f;
+  const bool zero = order_key(m) <= kKeyMin;
   const int64_t stride = (int64_t)gridDim.x * kReduceThreads;
   for (int64_t i = (int64_t)blockIdx.x * kReduceThreads + threadIdx.x; i < n; i += stride)
-    w[i] = m > -INFINITY ? w[i] * f : 0.0;
+    w[i] = zero ? 0.0 : w[i] * f;
 }
 
 }  // namespace

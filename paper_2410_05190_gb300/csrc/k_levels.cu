@@ -5,9 +5,10 @@
 // One thread-block cluster of 16 CTAs per slot: the call has no scratch and may not allocate,
 // and a cluster folds its CTAs' sums through distributed shared memory.  The pass reads 16
 // bytes per sample and slot; one CTA per slot, as before, kept a handful of loads in flight
-// on P of the 152 SMs (461 us for 5 slots of 2^18 samples, device time), 16 CTAs of 512
-// threads with four samples per thread in flight take 29 us.  Sums are FP64 in a fixed
-// order (deterministic).
+// on P of the 152 SMs (461 us for 5 slots of 2^18 samples, device time).  16 CTAs of 512
+// threads with the next four samples of a thread in flight during the adds of these, one FP64
+// add per sample, and the two sums of a warp folded by its two halves take 24 us (27 without
+// the loads ahead and with a fold each).  Sums are FP64 in a fixed order (deterministic).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -23,13 +24,15 @@ constexpr int kLevelThreads = 512;
 constexpr int kLevelCtas = 16;  // CTAs per slot: the largest cluster
 constexpr int kLevelUnroll = 4;
 constexpr int kMaxLevelSlots = 16;
+static_assert(kLevelCtas == 16 && kLevelThreads == 16 * 32, "half a warp folds the CTA's warps and the cluster's CTAs");
 
 struct LevelRef {
   double r[kMaxLevelSlots];
 };
 
 __global__ void __launch_bounds__(kLevelThreads) levels_kernel(int64_t n, const double* __restrict__ theta,
-                                                               const double* __restrict__ w, LevelRef ref,
+                                                               const double* __restrict__ w,
+                                                               const __grid_constant__ LevelRef ref,
                                                                double* __restrict__ out) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
@@ -40,14 +43,26 @@ __global__ void __launch_bounds__(kLevelThreads) levels_kernel(int64_t n, const 
   const double* x = theta + (int64_t)p * n;
   double below = 0.0, above = 0.0;
   constexpr int64_t kStride = (int64_t)kLevelCtas * kLevelThreads;
-  for (int64_t i0 = (int64_t)rank * kLevelThreads + threadIdx.x; i0 < n; i0 += kLevelUnroll * kStride) {
-    double wi[kLevelUnroll], xi[kLevelUnroll];
+  double wn[kLevelUnroll], xn[kLevelUnroll];
+  auto load = [&](int64_t i0) {
 #pragma unroll
     for (int u = 0; u < kLevelUnroll; ++u) {
       const int64_t i = i0 + u * kStride;
-      wi[u] = i < n ? w[i] : 0.0;
-      xi[u] = i < n ? x[i] : 0.0;
+      wn[u] = i < n ? w[i] : 0.0;
+      xn[u] = i < n ? x[i] : 0.0;
     }
+  };
+  int64_t i0 = (int64_t)rank * kLevelThreads + threadIdx.x;
+  load(i0);
+  while (i0 < n) {
+    double wi[kLevelUnroll], xi[kLevelUnroll];
+#pragma unroll
+    for (int u = 0; u < kLevelUnroll; ++u) {
+      wi[u] = wn[u];
+      xi[u] = xn[u];
+    }
+    i0 += kLevelUnroll * kStride;
+    load(i0);  // the next samples' loads fly during these ones' adds
 #pragma unroll
     for (int u = 0; u < kLevelUnroll; ++u) {
       // one FP64 add per sample: to the weight below or to the rest (a NaN is not below)
@@ -65,40 +80,28 @@ __global__ void __launch_bounds__(kLevelThreads) levels_kernel(int64_t n, const 
       above = lt ? above : sum;
     }
   }
-  double tot = below + above;
+  // the lower half of a warp folds the weight below, the upper half the total: one add a step
+  const int half = lane >> 4, hl = lane & 15;
+  const double tot = below + above;
+  double v = (half ? tot : below) + __shfl_xor_sync(0xffffffffu, half ? below : tot, 16);
+  auto fold16 = [&] {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    below += __shfl_xor_sync(0xffffffffu, below, o);
-    tot += __shfl_xor_sync(0xffffffffu, tot, o);
-  }
-  if (lane == 0) {
-    s_warp[0][threadIdx.x >> 5] = below;
-    s_warp[1][threadIdx.x >> 5] = tot;
-  }
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  };
+  fold16();
+  if (hl == 0) s_warp[half][threadIdx.x >> 5] = v;
   __syncthreads();
   if (threadIdx.x < 32) {
-    double v0 = lane < kLevelThreads / 32 ? s_warp[0][lane] : 0.0;
-    double v1 = lane < kLevelThreads / 32 ? s_warp[1][lane] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-      v1 += __shfl_xor_sync(0xffffffffu, v1, o);
-    }
-    if (lane == 0) {
-      s_cta[0] = v0;
-      s_cta[1] = v1;
-    }
+    v = s_warp[half][hl];
+    fold16();
+    if (hl == 0) s_cta[half] = v;
   }
   cluster.sync();
   if (rank == 0 && threadIdx.x < 32) {
-    double v0 = lane < kLevelCtas ? cluster.map_shared_rank(s_cta, lane)[0] : 0.0;
-    double v1 = lane < kLevelCtas ? cluster.map_shared_rank(s_cta, lane)[1] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-      v1 += __shfl_xor_sync(0xffffffffu, v1, o);
-    }
-    if (lane == 0) out[p] = v1 > 0.0 ? v0 / v1 : NAN;
+    v = cluster.map_shared_rank(s_cta, hl)[half];
+    fold16();
+    const double all = __shfl_sync(0xffffffffu, v, 16);
+    if (lane == 0) out[p] = all > 0.0 ? v / all : NAN;
   }
   cluster.sync();  // a CTA's shared memory outlives the reads of rank 0
 }

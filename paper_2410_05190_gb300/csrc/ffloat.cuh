@@ -5,6 +5,8 @@
 #pragma once
 #include <cstdint>
 
+#include "fpcvt.cuh"
+
 namespace mbis {
 
 // A value is an unevaluated pair hi + lo of floats.  Sums use Knuth's two-sum (exact), the
@@ -27,7 +29,7 @@ struct FFSum {
     h = s;
     l = __fadd_rn(l, e);
   }
-  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+  __device__ __forceinline__ double value() const { return to_double(h) + to_double(l); }
 };
 
 // (sh, sl) += (ch, cl) * (bh, bl)

@@ -169,8 +169,8 @@ __device__ __forceinline__ void fold_tile(const LikeArgs& a, int64_t tile, bool 
   for (int i = 0; i < kNumSlots; ++i) par[i] = (active && a.pos[i] >= 0) ? a.theta[(int64_t)a.pos[i] * a.n + s] : a.fixed[i];
   if (a.marg & MBIS_MARG_PHASE) par[kPhic] = 0.0;
   if (a.marg & MBIS_MARG_DISTANCE) par[kDl] = 1.0;
-  const bool valid = active && par[kMc] > 0.0 && par[kQ] > 0.0 && fabs(par[kChi1]) < 1.0 &&
-                     fabs(par[kChi2]) < 1.0 && par[kDl] > 0.0 && isfinite(par[kTc]) && isfinite(par[kPhic]);
+  const bool valid = active && is_positive(par[kMc]) && is_positive(par[kQ]) && is_below_one(par[kChi1]) &&
+                     is_below_one(par[kChi2]) && is_positive(par[kDl]) && is_finite(par[kTc]) && is_finite(par[kPhic]);
   int32_t kcut = 0;
   double A = 0.0;
   {
@@ -189,20 +189,14 @@ __device__ __forceinline__ void fold_tile(const LikeArgs& a, int64_t tile, bool 
     if constexpr (kFF) {
       float* pf = reinterpret_cast<float*>(sPC) + tid;
 #pragma unroll
-      for (int j = 0; j < kNumBasis; ++j) {
-        const float h = (float)pc.C[j];
-        pf[j * T] = h;
-        pf[(kNumBasis + 1 + j) * T] = (float)(pc.C[j] - (double)h);
-      }
-      const float h = (float)pc.cst;
-      pf[kNumBasis * T] = h;
-      pf[(2 * kNumBasis + 1) * T] = (float)(pc.cst - (double)h);
+      for (int j = 0; j < kNumBasis; ++j) split_float(pc.C[j], pf[j * T], pf[(kNumBasis + 1 + j) * T]);
+      split_float(pc.cst, pf[kNumBasis * T], pf[(2 * kNumBasis + 1) * T]);
     } else {
 #pragma unroll
       for (int j = 0; j < kNumBasis; ++j) sPC[j * T + tid] = pc.C[j];
       sPC[kNumBasis * T + tid] = pc.cst;
 #pragma unroll
-      for (int j = 0; j < kNumBasis - 1; ++j) sCF[j * T + tid] = (float)pc.C[j];
+      for (int j = 0; j < kNumBasis - 1; ++j) sCF[j * T + tid] = to_float(pc.C[j]);
     }
   }
   const double* my_pc = sPC + tid;

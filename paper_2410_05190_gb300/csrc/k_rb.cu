@@ -169,20 +169,20 @@ __global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
   auto par = [&](int slot) { return active && a.pos[slot] >= 0 ? a.theta[(int64_t)a.pos[slot] * a.n + s] : a.fixed[slot]; };
   const double mc = par(kMc), q = par(kQ), chi1 = par(kChi1), chi2 = par(kChi2);
   const double dl = (a.marg & MBIS_MARG_DISTANCE) ? 1.0 : par(kDl), tc = par(kTc), phic = par(kPhic);
-  const bool valid = active && mc > 0.0 && q > 0.0 && fabs(chi1) < 1.0 && fabs(chi2) < 1.0 && dl > 0.0 &&
-                     isfinite(tc) && isfinite(phic);
+  const bool valid = active && is_positive(mc) && is_positive(q) && is_below_one(chi1) && is_below_one(chi2) &&
+                     is_positive(dl) && is_finite(tc) && is_finite(phic);
   if (role == 0) {
     const double u = q + 2.0 + rcp_refined(q), u3 = u * u * u;
-    double y = (double)powf((float)u, 0.6f);
+    double y = to_double(powf(to_float(u), 0.6f));
     {
       const double y2 = y * y, y4 = y2 * y2;
-      y -= (y4 * y - u3) * (0.2 * (double)rcp_f32((float)y4));
+      y -= (y4 * y - u3) * (0.2 * to_double(rcp_f32(to_float(y4))));
     }
     const double am = kPi * kTsun * mc * y;
-    double a13 = (double)cbrtf((float)am);
+    double a13 = to_double(cbrtf(to_float(am)));
     {
       const double c2 = a13 * a13;
-      a13 -= (c2 * a13 - am) * ((1.0 / 3.0) * (double)rcp_f32((float)c2));
+      a13 -= (c2 * a13 - am) * ((1.0 / 3.0) * to_double(rcp_f32(to_float(c2))));
     }
     const double inv_a = rcp_refined(am);
     sm.mass[0][si] = u;
@@ -190,10 +190,10 @@ __global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
     sm.mass[2][si] = a13;
     sm.mass[3][si] = inv_a;
     const double fi = inv_a * (1.0 / 14.696938456699067);
-    const float kf = ceilf((float)(fi - a.f_lo) * rcp_f32((float)a.df));
+    const float kf = ceilf(to_float(fi - a.f_lo) * rcp_f32(to_float(a.df)));
     int32_t k = !(kf > 0.0f) ? 0 : (kf >= (float)a.n_bins ? a.n_bins : (int32_t)kf);
-    while (k > 0 && a.f_lo + (double)(k - 1) * a.df >= fi) --k;
-    while (k < a.n_bins && a.f_lo + (double)k * a.df < fi) ++k;
+    while (k > 0 && a.f_lo + to_double(k - 1) * a.df >= fi) --k;
+    while (k < a.n_bins && a.f_lo + to_double(k) * a.df < fi) ++k;
     sm.kcut[si] = valid ? k : 0;
   } else if (role == 1) {
     const double w = rcp_refined(1.0 + q);
@@ -206,10 +206,10 @@ __global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
     sm.pn[5][si] = t.phi7;
   } else if (role == 2) {
     const double x = mc * kTsun, x2 = x * x, x5 = x2 * x2 * x;
-    double z = (double)powf((float)x, 5.0f / 6.0f);
+    double z = to_double(powf(to_float(x), 5.0f / 6.0f));
     {
       const double z2 = z * z, z5 = z2 * z2 * z;
-      z -= (z5 * z - x5) * ((1.0 / 6.0) * (double)rcp_f32((float)z5));
+      z -= (z5 * z - x5) * ((1.0 / 6.0) * to_double(rcp_f32(to_float(z5))));
     }
     sm.amp[si] = 0.45643546458763845 * 0.46619407703541166 * z * rcp_refined(dl * kMpcSeconds);
   }
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
   {
     const double u = sm.mass[0][si], la = sm.mass[1][si], a13 = sm.mass[2][si], inv_a = sm.mass[3][si];
     const double pre = (3.0 / (256.0 * kPi)) * u;  // 3 / (128 eta) / (2 pi), turns
-    auto put = [&](int j, double C) { sm.dC[j][si] = (float)(C - (j < kNumBasis ? r.C0[j] : r.cst0)); };
+    auto put = [&](int j, double C) { sm.dC[j][si] = to_float(C - (j < kNumBasis ? r.C0[j] : r.cst0)); };
     if (role == 0) {
       const double pa = pre * inv_a;
       put(0, pa * inv_a * a13);                        // a^(-5/3)
@@ -353,16 +353,16 @@ __global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
       const int32_t k1 = __ldg(r.edges + n_mine + 1);
       float2 c_unused;
       const float2 rho1 = edge_rho(r.rec + kEdgeVec * (n_mine + 1), dCs, dcs, c_unused);
-      const double inv_w = 1.0 / ((double)(k1 - k0) * a.df);
-      const double sr1 = (double)(rho1.x - rho_n.x) * inv_w, si1 = (double)(rho1.y - rho_n.y) * inv_w;
+      const double inv_w = 1.0 / (to_double(k1 - k0) * a.df);
+      const double sr1 = to_double(rho1.x - rho_n.x) * inv_w, si1 = to_double(rho1.y - rho_n.y) * inv_w;
       const int64_t m = (int64_t)a.n_bins + 1;
       const double* T = r.prefix;
       const double a0r = T[kcut] - T[k0], a0i = T[m + kcut] - T[m + k0];
-      const double ofs = (double)k0 * a.df;
+      const double ofs = to_double(k0) * a.df;
       const double a1r = (T[2 * m + kcut] - T[2 * m + k0]) - ofs * a0r;
       const double a1i = (T[3 * m + kcut] - T[3 * m + k0]) - ofs * a0i;
-      zr64 += (double)rho_n.x * a0r - (double)rho_n.y * a0i + sr1 * a1r - si1 * a1i;
-      zi64 += (double)rho_n.x * a0i + (double)rho_n.y * a0r + sr1 * a1i + si1 * a1r;
+      zr64 += to_double(rho_n.x) * a0r - to_double(rho_n.y) * a0i + sr1 * a1r - si1 * a1i;
+      zi64 += to_double(rho_n.x) * a0i + to_double(rho_n.y) * a0r + sr1 * a1i + si1 * a1r;
     }
     const double amp = sm.amp[si];
     Z = amp * hypot(zr64, zi64);

@@ -31,7 +31,9 @@ __host__ __device__ inline void map_point(const TilingSpace& sp, double x, doubl
 }
 
 __device__ __forceinline__ bool in_space(const TilingSpace& sp, double x, double q) {
-  return x >= sp.x_lo && x < sp.x_hi && q >= sp.q_lo && q <= sp.q_hi;
+  // a NaN's key lies beyond every bound on its sign's side
+  const long long kx = order_key(x), kq = order_key(q);
+  return kx >= order_key(sp.x_lo) && kx < order_key(sp.x_hi) && kq >= order_key(sp.q_lo) && kq <= order_key(sp.q_hi);
 }
 
 // FP64 phase (turns) of a point's coefficients at frequency f
@@ -284,8 +286,8 @@ __device__ __forceinline__ void phase_coeffs_f32(float q, float chi1, float chi2
 // Per-sample set-up of the FP16 operand: the live-bin count from the total mass in FP64
 // (FP32 seed, one Newton step: the ISCO cut agrees with FP64 to the bin), the phase
 // coefficients in FP32, the inverse norm from the FP64 prefix table.  Bound by the FP64 pipe:
-// reciprocals from an FP32 seed, no library fmod or division, comparisons as integers (2^20
-// points: 157 us before, 104 now).
+// reciprocals from an FP32 seed, no library fmod or division (2^20 points: 157 us before, 104
+// so), comparisons and conversions on the integer pipe (65 us).
 struct FastSetup {
   float cf[kNumBasis - 1];
   int32_t kcut;
@@ -297,10 +299,10 @@ __device__ __forceinline__ FastSetup fast_setup(const TilingSpace& sp, const Til
   // the point's chirp mass and mass ratio (map_point), with one FP64 reciprocal: q and 1/q
   double mc = x;
   if (sp.mc_period > 0.0) {
-    const float turns = __fdividef((float)x, (float)sp.mc_period);
+    const float turns = __fdividef(to_float(x), to_float(sp.mc_period));
     double r;
     if (fabsf(turns) < 65536.0f) {  // the quotient's floor to one unit, then exact steps
-      r = fma(-(double)floorf(turns), sp.mc_period, x);
+      r = fma(-to_double(floorf(turns)), sp.mc_period, x);
       if (__double_as_longlong(r) < 0) r += sp.mc_period;
       if (order_key(r) >= order_key(sp.mc_period)) r -= sp.mc_period;
     } else {
@@ -312,21 +314,21 @@ __device__ __forceinline__ FastSetup fast_setup(const TilingSpace& sp, const Til
   const bool swap = order_key(q) < order_key(1.0);
   const double iq = rcp_refined(q), qp = swap ? iq : q;
   const double u = q + 2.0 + iq, u3 = u * u * u;   // (1 + q)^2 / q, the same for q and 1/q
-  double y = (double)powf((float)u, 0.6f);
+  double y = to_double(powf(to_float(u), 0.6f));
   const double y4 = (y * y) * (y * y);
-  y -= fma(y4, y, -u3) * (0.2 * (double)rcp_f32((float)y4));  // y^5 = u^3
+  y -= fma(y4, y, -u3) * (0.2 * to_double(rcp_f32(to_float(y4))));  // y^5 = u^3
   const double a = kPi * kTsun * mc * y;
   // grid points strictly below the ISCO: an FP32 estimate, then exact FP64 steps
   const double fi = rcp_refined(a) * (1.0 / 14.696938456699067);
   const long long fk = order_key(fi);
-  const float kf = ceilf((float)(fi - g.f_lo) * rcp_f32((float)g.df));
+  const float kf = ceilf(to_float(fi - g.f_lo) * rcp_f32(to_float(g.df)));
   int32_t k = !(kf > 0.0f) ? 0 : (kf >= (float)g.K ? g.K : (int32_t)kf);
-  while (k > 0 && order_key(fma((double)(k - 1), g.df, g.f_lo)) >= fk) --k;
-  while (k < g.K && order_key(fma((double)k, g.df, g.f_lo)) < fk) ++k;
+  while (k > 0 && order_key(fma(to_double(k - 1), g.df, g.f_lo)) >= fk) --k;
+  while (k < g.K && order_key(fma(to_double(k), g.df, g.f_lo)) < fk) ++k;
   o.kcut = k;
-  const float am = (float)a;
-  phase_coeffs_f32((float)qp, (float)sp.chi1, (float)sp.chi2, am, logf(am), cbrtf(am), o.cf);
-  o.inv_s = o.kcut > 0 ? rsqrtf((float)(g.w2sum[o.kcut] * g.inv_wref2)) : 0.f;
+  const float am = to_float(a);
+  phase_coeffs_f32(to_float(qp), to_float(sp.chi1), to_float(sp.chi2), am, logf(am), cbrtf(am), o.cf);
+  o.inv_s = o.kcut > 0 ? rsqrtf(to_float(g.w2sum[o.kcut] * g.inv_wref2)) : 0.f;
   return o;
 }
 

@@ -180,9 +180,9 @@ __global__ void __launch_bounds__(kTT, kCtasPerSm) loglike_mixed_time_kernel(Lik
 #pragma unroll
   for (int i = 0; i < kNumSlots; ++i)
     par[i] = (active && a.pos[i] >= 0) ? a.theta[(int64_t)a.pos[i] * a.n + s] : a.fixed[i];
-  const bool valid = active && par[kMc] > 0.0 && par[kQ] > 0.0 && fabs(par[kChi1]) < 1.0 &&
-                     fabs(par[kChi2]) < 1.0 && par[kDl] > 0.0 && isfinite(par[kTc]) && isfinite(par[kPhic]) &&
-                     isfinite(par[kRa]) && isfinite(par[kDec]) && isfinite(par[kPsi]) && isfinite(par[kIota]);
+  const bool valid = active && is_positive(par[kMc]) && is_positive(par[kQ]) && is_below_one(par[kChi1]) &&
+                     is_below_one(par[kChi2]) && is_positive(par[kDl]) && is_finite(par[kTc]) && is_finite(par[kPhic]) &&
+                     is_finite(par[kRa]) && is_finite(par[kDec]) && is_finite(par[kPsi]) && is_finite(par[kIota]);
   // exchange area in the A tiles' memory (free until the first rows are written):
   // [detector][sample] |P_d|, delay counter offset and step, |P_d|^2
   float* x_pm = reinterpret_cast<float*>(sm + Sh::kOffA);

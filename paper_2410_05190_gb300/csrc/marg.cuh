@@ -208,8 +208,8 @@ struct DistWindow {
 
 __device__ __forceinline__ DistWindow dist_window(double Z, double H, const DistConst& dc) {
   DistWindow d;
-  d.Z = (float)Z;
-  d.H = (float)H;
+  d.Z = to_float(Z);
+  d.H = to_float(H);
   d.window = false;
   d.wlo = 0.0f;
   d.whi = dc.span;
@@ -263,10 +263,10 @@ __device__ __forceinline__ double dist_finish(const DistWindow& d, LogSumExpF L,
     if (d.whi < dc.span && dist_node_g(d.hi, d.Z, d.H, d.u_ref, d.phi_ref) > L.m - kDistSkip)
       dist_rule_f(L, d.hi, dc.span - d.r_ref, 4, kGL8, x8, w8, d.Z, d.H, d.u_ref, d.phi_ref);
   }
-  const double u_ref = (double)d.u_ref;
+  const double u_ref = to_double(d.u_ref);
   const double g_ref =
-      dc.c0 - 3.0 * (dc.s_lo + (double)d.r_ref) + Z * u_ref - 0.5 * H * u_ref * u_ref + (double)d.phi_ref;
-  return g_ref + (double)L.m + (double)logf(L.acc);
+      dc.c0 - 3.0 * (dc.s_lo + to_double(d.r_ref)) + Z * u_ref - 0.5 * H * u_ref * u_ref + to_double(d.phi_ref);
+  return g_ref + to_double(L.m) + to_double(logf(L.acc));
 }
 
 __device__ __forceinline__ double log_distance_marginal_mixed(double Z, double H, const DistConst& dc,

@@ -15,6 +15,8 @@
 #include <cmath>
 #include <cstdint>
 
+#include "fpcvt.cuh"
+
 #ifdef __CUDACC__
 #define MBIS_HD __host__ __device__ __forceinline__
 #else
@@ -213,7 +215,7 @@ MBIS_HD float rcp_f32(float x) {
 }
 
 MBIS_HD double rcp_refined(double x) {
-  double r = (double)rcp_f32((float)x);
+  double r = to_double(rcp_f32(to_float(x)));
   r = fma(r, fma(-x, r, 1.0), r);
   return fma(r, fma(-x, r, 1.0), r);
 }
@@ -240,24 +242,24 @@ MBIS_HD SampleSetup sample_setup(double mc, double q, double chi1, double chi2, 
   const double w = rcp_refined(1.0 + q);
   const double u = q + 2.0 + rcp_refined(q), u3 = u * u * u;
   const double eta = q * w * w, dm = (q - 1.0) * w;
-  double y = (double)powf((float)u, 0.6f);
+  double y = to_double(powf(to_float(u), 0.6f));
   {
     const double y2 = y * y, y4 = y2 * y2;
-    y -= (y4 * y - u3) * (0.2 * (double)rcp_f32((float)y4));
+    y -= (y4 * y - u3) * (0.2 * to_double(rcp_f32(to_float(y4))));
   }
   const double a = kPi * kTsun * mc * y;
   const double la = log(a);
-  double a13 = (double)cbrtf((float)a);
+  double a13 = to_double(cbrtf(to_float(a)));
   {
     const double c2 = a13 * a13;
-    a13 -= (c2 * a13 - a) * ((1.0 / 3.0) * (double)rcp_f32((float)c2));
+    a13 -= (c2 * a13 - a) * ((1.0 / 3.0) * to_double(rcp_f32(to_float(c2))));
   }
   const double a23 = a13 * a13, inv_a = rcp_refined(a);
   const double x = mc * kTsun, x2 = x * x, x5 = x2 * x2 * x;
-  double z = (double)powf((float)x, 5.0f / 6.0f);
+  double z = to_double(powf(to_float(x), 5.0f / 6.0f));
   {
     const double z2 = z * z, z5 = z2 * z2 * z;
-    z -= (z5 * z - x5) * ((1.0 / 6.0) * (double)rcp_f32((float)z5));
+    z -= (z5 * z - x5) * ((1.0 / 6.0) * to_double(rcp_f32(to_float(z5))));
   }
   o.amp = 0.45643546458763845 * 0.46619407703541166 * z * rcp_refined(dl_mpc * kMpcSeconds);
 
@@ -278,10 +280,10 @@ MBIS_HD SampleSetup sample_setup(double mc, double q, double chi1, double chi2, 
   // the cut: an FP32 estimate of ceil((f_isco - f_lo) / df), then exact FP64 steps to the
   // first grid point at or above f_isco
   const double fi = inv_a * (1.0 / 14.696938456699067);
-  const float kf = ceilf((float)(fi - f_lo) * rcp_f32((float)df));
+  const float kf = ceilf(to_float(fi - f_lo) * rcp_f32(to_float(df)));
   int32_t k = !(kf > 0.0f) ? 0 : (kf >= (float)n_bins ? n_bins : (int32_t)kf);
-  while (k > 0 && f_lo + (double)(k - 1) * df >= fi) --k;
-  while (k < n_bins && f_lo + (double)k * df < fi) ++k;
+  while (k > 0 && f_lo + to_double(k - 1) * df >= fi) --k;
+  while (k < n_bins && f_lo + to_double(k) * df < fi) ++k;
   o.kcut = k;
   return o;
 }

@@ -151,8 +151,9 @@ struct Branches {
 // Enqueue one step on b->stream, under capture.  The events' draws and orders depend on the
 // counters alone, and their reductions on the likelihoods alone, so they run on branches side
 // by side: a draw or a reduction of 2^14 .. 2^17 samples is a chain of FP64 latencies on part
-// of the GPU (a step of 8 events of 2^14 .. 2^17 samples takes
-// 12.25 ms with them one after another, 12.01 ms on branches).  Events that share a context share its reduction scratch and so a branch.
+// of the GPU (a step of 8 events of such sizes takes 12.25 ms with them one after another,
+// 12.01 ms on branches).  Events that share a context share its reduction scratch and so a
+// branch.
 mbis_status enqueue_step(mbis_batch* b, Branches& br) {
   std::vector<cudaStream_t> on(b->n);
   std::unordered_map<const mbis_ctx*, cudaStream_t> taken;

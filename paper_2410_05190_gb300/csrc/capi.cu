@@ -539,7 +539,10 @@ mbis_status mbis::ess_issue(mbis_ctx* c, EssState* st, const EssBuffers& buf, cu
   CU_TRY(c, launch_draw(da, s));
   mbis_status r = mbis_loglike(c, nb, buf.theta, buf.loglike, s);
   if (r != MBIS_OK) return r;
-  CU_TRY(c, launch_reduce(nb, buf.loglike, buf.log_prior, buf.log_q, st->refit ? buf.weights : nullptr, c->red, s));
+  if (st->refit)
+    CU_TRY(c, launch_reduce_ordered(nb, buf.loglike, buf.log_prior, buf.log_q, buf.weights, c->red, s));
+  else
+    CU_TRY(c, launch_reduce(nb, buf.loglike, buf.log_prior, buf.log_q, nullptr, c->red, s));
   CU_TRY(c, cudaMemcpyAsync(c->h_result, c->red.result, sizeof(double) * 4, cudaMemcpyDeviceToHost, s));
   CU_TRY(c, cudaMemcpyAsync(c->h_result + 4, c->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   if (st->refit) {

@@ -185,7 +185,7 @@ cudaError_t launch_loglike_mixed_batch(const LikeArgs* args, const BatchItem* it
                                       int32_t grid, bool ff, int32_t tile, cudaStream_t s);
 int32_t batch_ctas_per_sm(int32_t tile);
 
-// two-pass weight reduction; partials / counter / result are device scratch
+// weight reduction; partials / counter / result are device scratch
 struct ReduceScratch {
   double* partials;       // [3 * kReduceBlocks]: (m_b, S1_b, S2_b) per CTA
   unsigned int* counter;  // [1], zero between calls
@@ -193,6 +193,8 @@ struct ReduceScratch {
 };
 cudaError_t launch_reduce(int64_t n, const double* loglike, const double* logp, const double* logq,
                           double* weights, const ReduceScratch& scr, cudaStream_t s);
+cudaError_t launch_reduce_ordered(int64_t n, const double* loglike, const double* logp, const double* logq,
+                                  double* weights, const ReduceScratch& scr, cudaStream_t s);
 
 // waveform helpers (FP64): strain of n_par parameter vectors, and inner products
 cudaError_t launch_waveforms(int32_t n_par, const double* par /*[n_par][11] device*/, int32_t n_det, int32_t n_bins,

@@ -14,12 +14,14 @@
 //     cosine and the Cholesky sums (a normal's error is 2.8e-17 rms and 1.2e-15 at most over
 //     3 10^6 draws, against 2.4e-16 and 2.9e-15 in FP64) -- which leaves FP64 a conversion and
 //     a multiply-add per slot;
-//   * contexts of MBIS_MIXED: the library's FP64 functions, whose last bits these samples have
-//     always had.  The mixed likelihoods round in FP32, so a sample one FP64 ulp away can round
-//     to another log L (by up to 6e-8 of its spread, seen in 2 of 50 batches): with this choice
-//     a seed keeps its results.
+//   * contexts of MBIS_MIXED: the library's FP64 functions for normals, density and prior, whose
+//     last bits these samples have always had.  The mixed likelihoods round in FP32, so a sample
+//     one FP64 ulp away can round to another log L (by up to 6e-8 of its spread, seen in 2 of 50
+//     batches), and a refit feeds such a difference back: with this choice a seed keeps its
+//     results.  (The sum of squares takes explicit multiply-adds: an unrolled chain of sums is
+//     re-associated when it is contracted.)
 // Measured on a GB300 (device time): 2^18 samples of 11 slots 429 us before and 58 us fixed;
-// 2^16 of 5 slots 50 us before, 10 us fixed and 37 us library.
+// 2^16 of 5 slots 50 us before, 10 us fixed.
 #include <algorithm>
 #include <cmath>
 
@@ -35,6 +37,7 @@ constexpr int kDrawThreads = 128;
 
 struct DrawConsts {
   double lp_const;          // the prior's log-normalisation, all slots
+  double lpc[kMaxP];        // and slot by slot
   double row_scale[kMaxP];  // 2^(E_p - 56), every element of row p of scale * L below 2^E_p
   Pair28 chol[kMaxP * (kMaxP + 1) / 2];  // those elements in that unit, row by row
   double chol64[kMaxP * (kMaxP + 1) / 2];  // and in FP64
@@ -124,6 +127,7 @@ __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawCons
   Pair28 z[P + 1];
   double zd[P + 1];
   double half_zz = 0.0;  // sum z^2 / 2
+  double lp = 0.0;       // the log prior (library arithmetic)
   {
     int64_t half_zz54 = 0;  // unit 2^-54
 #pragma unroll
@@ -138,16 +142,22 @@ __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawCons
           const int64_t t = box_muller(tb, w.v[2 * h], w.v[2 * h + 1], z[p], z[p + 1]);
           half_zz54 += p + 1 < P ? (t + 8) >> 4 : (mul28(z[p], z[p], 0) + 4) >> 3;
         } else {
-          const double l = log(uniform64(w.v[2 * h])), r = sqrt(-2.0 * l);
+          const double r = sqrt(-2.0 * log(uniform64(w.v[2 * h])));
           double sn, cs;
           sincospi(2.0 * uniform64(w.v[2 * h + 1]), &sn, &cs);
           zd[p] = r * cs;
           zd[p + 1] = r * sn;
-          half_zz = p + 1 < P ? half_zz - l : fma(0.5 * zd[p], zd[p], half_zz);
         }
       }
     }
-    if constexpr (kFixed) half_zz = (double)half_zz54 * 0x1p-54;
+    if constexpr (kFixed) {
+      half_zz = (double)half_zz54 * 0x1p-54;
+    } else {
+      double zz = 0.0;
+#pragma unroll
+      for (int p = 0; p < P; ++p) zz = __fma_rn(zd[p], zd[p], zz);
+      half_zz = 0.5 * zz;
+    }
   }
   double mc = 0.0, q = 0.0;
   bool inside = true;
@@ -172,10 +182,24 @@ __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawCons
     if (id == kRa || id == kPhic) x = wrap_period(x, kTwoPi);
     if (id == kPsi) x = wrap_period(x, kPi);
     a.theta[(int64_t)p * a.n + i] = x;
-    if (id == kRa || id == kPhic || id == kPsi) continue;
+    if (id == kRa || id == kPhic || id == kPsi) {
+      if constexpr (!kFixed) lp += k.lpc[p];
+      continue;
+    }
     inside = inside && !is_nan(x) && order_key(x) >= order_key(a.lo[p]) && order_key(x) <= order_key(a.hi[p]);
     if (id == kMc) mc = x;
     if (id == kQ) q = x;
+    if constexpr (!kFixed) {
+      if (id == kDec)
+        lp += log(cos(x)) + k.lpc[p];
+      else if (id == kIota)
+        lp += log(sin(x)) + k.lpc[p];
+      else if (id == kDl)
+        lp += 2.0 * log(x) + k.lpc[p];
+      else
+        lp += k.lpc[p];
+      continue;
+    }
     if (id == kDec || id == kIota) {
       int64_t co, si;
       trig_of(tb, angle_turns(inside ? x : 1.0), co, si);
@@ -186,8 +210,15 @@ __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawCons
     }
     if (id == kDl) log_sum50 += log_of(tb, inside ? x : 1.0) >> 1;
   }
+  // |d(m1, m2)/d(Mc, q)| = Mc (1 + q)^(2/5) q^(-6/5)
+  if constexpr (!kFixed) {
+    if ((a.flags & MBIS_PRIOR_M1M2) && inside)
+      lp += 0.4 * log(mc * mc * sqrt(mc) * (1.0 + q) / (q * q * q)) - a.log_mass_norm;
+    if (a.logp) a.logp[i] = inside ? lp : -INFINITY;
+    if (a.logq) a.logq[i] = a.log_q_const - half_zz;
+    return;
+  }
   if ((a.flags & MBIS_PRIOR_M1M2) && inside) {
-    // |d(m1, m2)/d(Mc, q)| = Mc (1 + q)^(2/5) q^(-6/5)
     const int64_t lq = log_of(tb, q);
     log_sum50 += (log_of(tb, mc) + __mul64hi(log_of(tb, 1.0 + q), 0x6666666666666666ll) - lq -
                   __mul64hi(lq, 0x3333333333333333ll)) >> 2;
@@ -215,15 +246,14 @@ cudaError_t launch_draw(const DrawArgs& a, cudaStream_t s) {
     const int id = a.ids[p];
     const double lo = a.lo[p], hi = a.hi[p];
     switch (id) {
-      case kRa: case kPhic: k.lp_const -= log(kTwoPi); break;
-      case kPsi: k.lp_const -= log(kPi); break;
-      case kDec: k.lp_const -= log(sin(hi) - sin(lo)); break;
-      case kIota: k.lp_const -= log(cos(lo) - cos(hi)); break;
-      case kDl: k.lp_const += log(3.0) - log(hi * hi * hi - lo * lo * lo); break;
-      default:
-        if (!((a.flags & MBIS_PRIOR_M1M2) && (id == kMc || id == kQ))) k.lp_const -= log(hi - lo);
-        break;
+      case kRa: case kPhic: k.lpc[p] = -log(kTwoPi); break;
+      case kPsi: k.lpc[p] = -log(kPi); break;
+      case kDec: k.lpc[p] = -log(sin(hi) - sin(lo)); break;
+      case kIota: k.lpc[p] = -log(cos(lo) - cos(hi)); break;
+      case kDl: k.lpc[p] = log(3.0) - log(hi * hi * hi - lo * lo * lo); break;
+      default: k.lpc[p] = (a.flags & MBIS_PRIOR_M1M2) && (id == kMc || id == kQ) ? 0.0 : -log(hi - lo); break;
     }
+    k.lp_const += k.lpc[p];
     // the row of scale * L in fixed point, in units of its largest element; a factor that is
     // not finite leaves its slot's draws not finite
     double row[kMaxP];

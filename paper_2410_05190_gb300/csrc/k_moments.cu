@@ -6,23 +6,23 @@
 // [-period/2, period/2) around ref), the kernel accumulates sum w d and sum w d d^T in FP64;
 // offsets keep the sums well conditioned for parameters measured to ~1e-5 relative.
 //
-// What bounds it is the FP64 pipe: 1 + 2 P + P (P + 1) / 2 multiply-adds and P subtractions
-// per sample (13 us for 5 slots of 2^18 samples).  One instantiation per slot count keeps
-// every sum in registers (with a run-time count the sums lived in local memory).  The sums
-// of a warp fold by recursive halving -- each step a lane keeps half of its sums and takes
-// its partner's part of them, so M sums cost M adds instead of 5 M -- then the CTA's warps
-// through shared memory; per-CTA partials go to device scratch and the last CTA folds them
-// in a fixed order with all its threads.  Measured on a GB300 (device time, 5 slots): 83 us
-// at 2^18 samples and 48 us at 2^16 before, 26 and 14 us now.
+// What bounds it is the FP64 pipe: 1 + 2 P + P (P + 1) / 2 multiply-adds and 2 P other
+// operations per sample (15 us for 5 slots of 2^18 samples), and at the end the CTAs' sums added
+// one after another (304 dependent adds, 10 us).  That order, like the tree over a CTA's threads,
+// is part of the result: a refit feeds the moments back into draws whose FP32 likelihoods turn a
+// last bit into 1e-6 of the fitted Gaussian.  One instantiation per slot count keeps every sum in
+// registers (with a run-time count the sums lived in local memory).  The sums of a warp fold by
+// recursive halving -- each step a lane keeps half of its sums and takes its partner's part of
+// them, so M sums cost M adds instead of 5 M, in the tree's pairs.  The posterior stage of 2^18
+// samples (weights, moments, levels; GB300): 667 us before, 133 now, 119 with an order of its own.
 #include "fpkey.cuh"
 #include "internal.h"
 
 namespace mbis {
 namespace {
 
-constexpr int kMomThreads = 256;
-constexpr int kMomBlocks = 152;  // one per SM: the fold's cost grows with the warps
-constexpr int kMomWarps = kMomThreads / 32;
+constexpr int kMomThreads = 128;
+constexpr int kMomBlocks = 304;  // two per SM
 
 __host__ __device__ constexpr int moment_sums(int P) { return 1 + P + P * (P + 1) / 2; }
 
@@ -55,7 +55,7 @@ struct WarpFold {
 };
 
 template <int P>
-__global__ void __launch_bounds__(kMomThreads, 1) moments_kernel(int64_t n, const double* theta, const double* w,
+__global__ void __launch_bounds__(kMomThreads, 2) moments_kernel(int64_t n, const double* theta, const double* w,
                                                                  MomentArgs ma, double* partials,
                                                                  unsigned int* counter, double* out) {
   constexpr int nm = moment_sums(P);  // sum of weights, first moments, upper triangle
@@ -89,8 +89,8 @@ __global__ void __launch_bounds__(kMomThreads, 1) moments_kernel(int64_t n, cons
       d[p] -= ma.ref[p];
       const double T = ma.period[p];
       if (T > 0.0) {
-        // a division and a floor only for an offset outside [-T/2, T/2)
-        const long long k = order_key(d[p]), h = order_key(0.5 * T);
+        // a division and a floor only for an offset that they can move
+        const long long k = order_key(d[p]), h = order_key(0.4375 * T);
         if (k < -h || k >= h) d[p] -= T * floor(d[p] / T + 0.5);
       }
     }
@@ -100,7 +100,8 @@ __global__ void __launch_bounds__(kMomThreads, 1) moments_kernel(int64_t n, cons
 #pragma unroll
     for (int p = 0; p < P; ++p) {
       wd[p] = wi * d[p];
-      acc[m++] += wd[p];
+      acc[m] = fma(wi, d[p], acc[m]);
+      ++m;
     }
 #pragma unroll
     for (int p = 0; p < P; ++p)
@@ -110,39 +111,45 @@ __global__ void __launch_bounds__(kMomThreads, 1) moments_kernel(int64_t n, cons
         ++m;
       }
   }
-  __shared__ double sh[kMomWarps][nm];
+  // the CTA's sums: a binary tree over its threads, the upper half of them adding into the lower
+  __shared__ double sh[nm][kMomThreads / 2];
   __shared__ bool last;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int base = 0, count = nm;
-  WarpFold<nm, 16>::run(acc, lane, base, count, sh[warp]);
-  __syncthreads();
-  for (int m = threadIdx.x; m < nm; m += kMomThreads) {
-    double s = sh[0][m];
+  const int t = threadIdx.x;
 #pragma unroll
-    for (int k = 1; k < kMomWarps; ++k) s += sh[k][m];
-    partials[(int64_t)blockIdx.x * nm + m] = s;
+  for (int h = kMomThreads / 2; h >= 32; h >>= 1) {
+    if (h < kMomThreads / 2) __syncthreads();
+    if (t >= h && t < 2 * h)
+#pragma unroll
+      for (int m = 0; m < nm; ++m) sh[m][t - h] = acc[m];
+    __syncthreads();
+    if (t < h)
+#pragma unroll
+      for (int m = 0; m < nm; ++m) acc[m] += sh[m][t];
+  }
+  if (t < 32) {
+    int base = 0, count = nm;
+    WarpFold<nm, 16>::run(acc, t, base, count, partials + (int64_t)blockIdx.x * nm);
   }
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  if (t == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
   __syncthreads();
   if (last) {
-    // kPer threads per sum, each over a strided share of the CTAs' partials
-    constexpr int kPer = kMomThreads / nm < kMomWarps ? kMomThreads / nm : kMomWarps;
-    const int m = threadIdx.x % nm, part = threadIdx.x / nm;
-    if (part < kPer) {
+    // one thread per sum, the CTAs one after another
+    if (t < nm) {
       double s = 0.0;
-      for (int b = part; b < (int)gridDim.x; b += kPer) s += __ldcg(partials + (int64_t)b * nm + m);
-      sh[part][m] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < nm) {
-      double s = sh[0][threadIdx.x];
+      constexpr int kLoads = 16;
+      for (int b0 = 0; b0 < (int)gridDim.x; b0 += kLoads) {
+        double v[kLoads];
 #pragma unroll
-      for (int k = 1; k < kPer; ++k) s += sh[k][threadIdx.x];
-      out[threadIdx.x] = s;
+        for (int k = 0; k < kLoads; ++k)
+          v[k] = b0 + k < (int)gridDim.x ? __ldcg(partials + (int64_t)(b0 + k) * nm + t) : 0.0;
+#pragma unroll
+        for (int k = 0; k < kLoads; ++k) s += v[k];
+      }
+      out[t] = s;
     }
-    if (threadIdx.x == 0) *counter = 0u;
+    if (t == 0) *counter = 0u;
   }
 }
 

@@ -20,13 +20,12 @@
 // sweep).
 //
 // A CTA takes 64 samples, two per lane in packed FP32 (one record read and one instruction for
-// both), and its eight warps share the chunks, the per-sample set-up (its independent parts on
-// different warps) and the nodes of the distance marginal.  Bound by instruction issue (12 per
-// sample and edge beside 2 sine/cosine results); one sample per thread over all edges, the
-// version before, issued 21 and left a 2^16-sample batch two CTAs of 256 threads per SM.
-// Measured on a GB300 on two BNS events (1.8 10^3 and 0.8 10^3 edges): 2^12 samples 160 and
-// 113 us before, 78 and 49 now; 2^16 254 and 165, 189 and 135; 2^20 2.68 and 1.44 ms, 2.49 and
-// 1.39 ms.
+// both), and its eight warps share the chunks and the nodes of the distance marginal; a sample's
+// chunk sums are then added in order by two threads, so that its log L has the bits of one
+// thread's sweep.  Bound by instruction issue (12 per sample and edge beside 2 sine/cosine
+// results) and the FP64 set-up; one sample per thread over all edges, the version before, issued
+// 21 and left a 2^16-sample batch two CTAs of 256 threads per SM.  A run to a target ESS (GB300,
+// the same reductions and moments): 1.71 to 1.93 ms before, 1.53 to 1.59 now.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -145,12 +144,10 @@ __device__ __forceinline__ float2 edge_rho(const float4* __restrict__ e, const f
 }
 
 struct RbSmem {
-  double mass[4][kRbTile];   // u, ln a, a^(1/3), 1 / a
-  double pn[6][kRbTile];
   double amp[kRbTile];
   float dC[kNumBasis + 1][kRbTile];
   int32_t kcut[kRbTile];
-  float part[kRbWarps][4][kRbTile];  // per warp: re (hi, lo), im (hi, lo)
+  float part[2][kRbTile];            // the imaginary sum (hi, lo)
   float dist[6][kRbTile];            // the distance rule: lo, hi, Z, H, u_ref, phi_ref
   int32_t nodes[kRbTile];            // its nodes: 48, 192 without a window, 0 outside the model
   float g[2][kGL48][kRbTile];        // 48 node values at a time, two rounds in turn
@@ -162,7 +159,7 @@ __global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t s0 = (int64_t)blockIdx.x * kRbTile;
 
-  // ---- per-sample set-up (sample_setup of physics.cuh, its parts on different warps)
+  // ---- per-sample set-up
   const int si = threadIdx.x & (kRbTile - 1), role = threadIdx.x / kRbTile;
   const int64_t s = s0 + si;
   const bool active = s < a.n;
@@ -171,69 +168,23 @@ __global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
   const double dl = (a.marg & MBIS_MARG_DISTANCE) ? 1.0 : par(kDl), tc = par(kTc), phic = par(kPhic);
   const bool valid = active && is_positive(mc) && is_positive(q) && is_below_one(chi1) && is_below_one(chi2) &&
                      is_positive(dl) && is_finite(tc) && is_finite(phic);
-  if (role == 0) {
-    const double u = q + 2.0 + rcp_refined(q), u3 = u * u * u;
-    double y = to_double(powf(to_float(u), 0.6f));
-    {
-      const double y2 = y * y, y4 = y2 * y2;
-      y -= (y4 * y - u3) * (0.2 * to_double(rcp_f32(to_float(y4))));
-    }
-    const double am = kPi * kTsun * mc * y;
-    double a13 = to_double(cbrtf(to_float(am)));
-    {
-      const double c2 = a13 * a13;
-      a13 -= (c2 * a13 - am) * ((1.0 / 3.0) * to_double(rcp_f32(to_float(c2))));
-    }
-    const double inv_a = rcp_refined(am);
-    sm.mass[0][si] = u;
-    sm.mass[1][si] = log(am);
-    sm.mass[2][si] = a13;
-    sm.mass[3][si] = inv_a;
-    const double fi = inv_a * (1.0 / 14.696938456699067);
-    const float kf = ceilf(to_float(fi - a.f_lo) * rcp_f32(to_float(a.df)));
-    int32_t k = !(kf > 0.0f) ? 0 : (kf >= (float)a.n_bins ? a.n_bins : (int32_t)kf);
-    while (k > 0 && a.f_lo + to_double(k - 1) * a.df >= fi) --k;
-    while (k < a.n_bins && a.f_lo + to_double(k) * a.df < fi) ++k;
-    sm.kcut[si] = valid ? k : 0;
-  } else if (role == 1) {
-    const double w = rcp_refined(1.0 + q);
-    const PNTerms t = pn_terms(q * w * w, (q - 1.0) * w, 0.5 * (chi1 + chi2), 0.5 * (chi1 - chi2));
-    sm.pn[0][si] = t.phi2;
-    sm.pn[1][si] = t.phi3;
-    sm.pn[2][si] = t.phi4;
-    sm.pn[3][si] = t.c5;
-    sm.pn[4][si] = t.a6;
-    sm.pn[5][si] = t.phi7;
-  } else if (role == 2) {
-    const double x = mc * kTsun, x2 = x * x, x5 = x2 * x2 * x;
-    double z = to_double(powf(to_float(x), 5.0f / 6.0f));
-    {
-      const double z2 = z * z, z5 = z2 * z2 * z;
-      z -= (z5 * z - x5) * ((1.0 / 6.0) * to_double(rcp_f32(to_float(z5))));
-    }
-    sm.amp[si] = 0.45643546458763845 * 0.46619407703541166 * z * rcp_refined(dl * kMpcSeconds);
-  }
-  __syncthreads();
-  {
-    const double u = sm.mass[0][si], la = sm.mass[1][si], a13 = sm.mass[2][si], inv_a = sm.mass[3][si];
-    const double pre = (3.0 / (256.0 * kPi)) * u;  // 3 / (128 eta) / (2 pi), turns
-    auto put = [&](int j, double C) { sm.dC[j][si] = to_float(C - (j < kNumBasis ? r.C0[j] : r.cst0)); };
-    if (role == 0) {
-      const double pa = pre * inv_a;
-      put(0, pa * inv_a * a13);                        // a^(-5/3)
-      put(1, pa * sm.pn[0][si]);                       // a^(-1)
-      put(2, pa * sm.pn[1][si] * a13);                 // a^(-2/3)
-    } else if (role == 1) {
-      const double a23 = a13 * a13;
-      put(3, pre * inv_a * sm.pn[2][si] * a23);        // a^(-1/3)
-      put(7, pre * sm.pn[5][si] * a23);
-      put(8, tc);
-    } else if (role == 2) {
-      put(5, pre * a13 * (sm.pn[4][si] - 6848.0 / 63.0 * la));
-      put(6, -pre * a13 * (6848.0 / 63.0));
+  // One thread per sample and straight-line code: shared among warps, or past a branch, C - C0
+  // loses its contraction, a last FP64 bit that turns a last FP32 bit of dC in one sample of
+  // 7 10^4 -- enough to move a refitted proposal by 1e-7.  The warps that do it rotate, so that
+  // the CTAs of an SM do not queue on the same SM quarters.
+  if (role == (int)(blockIdx.x / 152 & 3)) {
+    if (valid) {
+      const SampleSetup ss = sample_setup(mc, q, chi1, chi2, tc, phic, dl, a.f_lo, a.df, a.n_bins);
+#pragma unroll
+      for (int j = 0; j < kNumBasis; ++j) sm.dC[j][si] = to_float(ss.pc.C[j] - r.C0[j]);
+      sm.dC[kNumBasis][si] = to_float(ss.pc.cst - r.cst0);
+      sm.kcut[si] = ss.kcut;
+      sm.amp[si] = ss.amp;
     } else {
-      put(4, pre * sm.pn[3][si]);                      // ln f
-      put(kNumBasis, phic * (-1.0 / kTwoPi) - 0.125 + pre * sm.pn[3][si] * (1.0 + la));
+#pragma unroll
+      for (int j = 0; j <= kNumBasis; ++j) sm.dC[j][si] = 0.f;
+      sm.kcut[si] = 0;
+      sm.amp[si] = 0.0;
     }
   }
   __syncthreads();
@@ -262,47 +213,52 @@ __global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
     }
     nfull[h] = lo;
   }
-  const int32_t n_max = __reduce_max_sync(0xffffffffu, max(nfull[0], nfull[1]));
-  FFSum zr_all[2], zi_all[2];  // chunk sums, scaled by 1 / scale
-  for (int32_t e = kRbChunk * warp; e + kRbChunk <= n_max; e += kRbChunk * kRbWarps) {
-    float2 zr = f2(0.f), zi = f2(0.f);
-    const float4* rec = r.rec + kEdgeVec * e;
+  // The warps evaluate 48 chunks at a time; two threads per sample then add its chunk sums in
+  // order, as a pair (the real and the imaginary ones, scaled by 1 / scale).
+  const int32_t n_chunks = __reduce_max_sync(0xffffffffu, max(nfull[0], nfull[1])) / kRbChunk;
+  const int32_t my_chunks = nfull[warp & 1] / kRbChunk;  // of sample si
+  FFSum z_all;
+  for (int32_t c0 = 0; c0 < n_chunks; c0 += kGL48) {
+    const int32_t nc = min(n_chunks - c0, (int32_t)kGL48);
+    for (int32_t c = warp; c < nc; c += kRbWarps) {
+      float2 zr = f2(0.f), zi = f2(0.f);
+      const float4* rec = r.rec + kEdgeVec * kRbChunk * (c0 + c);
 #pragma unroll
-    for (int j = 0; j < kRbChunk; ++j) {
-      const float4 r0 = __ldg(rec + kEdgeVec * j), r1 = __ldg(rec + kEdgeVec * j + 1), r2 = __ldg(rec + kEdgeVec * j + 2);
-      float2 t = __ffma2_rn(dC[0], f2(r0.z), dcst);
-      t = __ffma2_rn(dC[1], f2(r0.w), t);
-      t = __ffma2_rn(dC[2], f2(r1.x), t);
-      t = __ffma2_rn(dC[3], f2(r1.y), t);
-      t = __ffma2_rn(dC[4], f2(r1.z), t);
-      t = __ffma2_rn(dC[5], f2(r1.w), t);
-      t = __ffma2_rn(dC[6], f2(r2.x), t);
-      t = __ffma2_rn(dC[7], f2(r2.y), t);
-      t = __ffma2_rn(dC[8], f2(r2.z), t);
-      // the nearest integer removed, as edge_rho does
-      const float2 n = __fadd2_rn(__fadd2_rn(t, f2(12582912.0f)), f2(-12582912.0f));
-      const float2 ang = __fmul2_rn(f2(-kTwoPiF), __fadd2_rn(t, make_float2(-n.x, -n.y)));
-      float2 sn, co;
-      __sincosf(ang.x, &sn.x, &co.x);
-      __sincosf(ang.y, &sn.y, &co.y);
-      zr = __ffma2_rn(co, f2(r0.x), __ffma2_rn(sn, f2(-r0.y), zr));
-      zi = __ffma2_rn(co, f2(r0.y), __ffma2_rn(sn, f2(r0.x), zi));
+      for (int j = 0; j < kRbChunk; ++j) {
+        const float4 r0 = __ldg(rec + kEdgeVec * j), r1 = __ldg(rec + kEdgeVec * j + 1), r2 = __ldg(rec + kEdgeVec * j + 2);
+        float2 t = __ffma2_rn(dC[0], f2(r0.z), dcst);
+        t = __ffma2_rn(dC[1], f2(r0.w), t);
+        t = __ffma2_rn(dC[2], f2(r1.x), t);
+        t = __ffma2_rn(dC[3], f2(r1.y), t);
+        t = __ffma2_rn(dC[4], f2(r1.z), t);
+        t = __ffma2_rn(dC[5], f2(r1.w), t);
+        t = __ffma2_rn(dC[6], f2(r2.x), t);
+        t = __ffma2_rn(dC[7], f2(r2.y), t);
+        t = __ffma2_rn(dC[8], f2(r2.z), t);
+        // the nearest integer removed, as edge_rho does
+        const float2 n = __fadd2_rn(__fadd2_rn(t, f2(12582912.0f)), f2(-12582912.0f));
+        const float2 ang = __fmul2_rn(f2(-kTwoPiF), __fadd2_rn(t, make_float2(-n.x, -n.y)));
+        float2 sn, co;
+        __sincosf(ang.x, &sn.x, &co.x);
+        __sincosf(ang.y, &sn.y, &co.y);
+        zr = __ffma2_rn(co, f2(r0.x), __ffma2_rn(sn, f2(-r0.y), zr));
+        zi = __ffma2_rn(co, f2(r0.y), __ffma2_rn(sn, f2(r0.x), zi));
+      }
+      sm.g[0][c][lane] = zr.x;
+      sm.g[0][c][lane + 32] = zr.y;
+      sm.g[1][c][lane] = zi.x;
+      sm.g[1][c][lane + 32] = zi.y;
     }
-    if (e + kRbChunk <= nfull[0]) {
-      zr_all[0].add(zr.x);
-      zi_all[0].add(zi.x);
+    __syncthreads();
+    if (role < 2) {
+      const int32_t m = min(my_chunks - c0, (int32_t)kGL48);
+      for (int32_t c = 0; c < m; ++c) z_all.add(sm.g[role][c][si]);
     }
-    if (e + kRbChunk <= nfull[1]) {
-      zr_all[1].add(zr.y);
-      zi_all[1].add(zi.y);
-    }
+    __syncthreads();
   }
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    sm.part[warp][0][lane + 32 * h] = zr_all[h].h;
-    sm.part[warp][1][lane + 32 * h] = zr_all[h].l;
-    sm.part[warp][2][lane + 32 * h] = zi_all[h].h;
-    sm.part[warp][3][lane + 32 * h] = zi_all[h].l;
+  if (role == 1) {
+    sm.part[0][si] = z_all.h;
+    sm.part[1][si] = z_all.l;
   }
   // ---- one thread per sample: the edges after its last whole chunk, the bin holding its cut,
   // the sums of the warps in order
@@ -334,14 +290,9 @@ __global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
   }
   __syncthreads();
   if (role == 0) {
-    FFSum sr, sc;
-#pragma unroll
-    for (int w = 0; w < kRbWarps; ++w) {
-      sr.add(sm.part[w][0][si]);
-      sr.l = __fadd_rn(sr.l, sm.part[w][1][si]);
-      sc.add(sm.part[w][2][si]);
-      sc.l = __fadd_rn(sc.l, sm.part[w][3][si]);
-    }
+    FFSum sr = z_all, sc;
+    sc.h = sm.part[0][si];
+    sc.l = sm.part[1][si];
     sr.add(zr);
     sc.add(zi);
     double zr64 = sr.value() * r.scale, zi64 = sc.value() * r.scale;
@@ -353,16 +304,16 @@ __global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
       const int32_t k1 = __ldg(r.edges + n_mine + 1);
       float2 c_unused;
       const float2 rho1 = edge_rho(r.rec + kEdgeVec * (n_mine + 1), dCs, dcs, c_unused);
-      const double inv_w = 1.0 / (to_double(k1 - k0) * a.df);
-      const double sr1 = to_double(rho1.x - rho_n.x) * inv_w, si1 = to_double(rho1.y - rho_n.y) * inv_w;
+      const double inv_w = 1.0 / ((double)(k1 - k0) * a.df);
+      const double sr1 = (double)(rho1.x - rho_n.x) * inv_w, si1 = (double)(rho1.y - rho_n.y) * inv_w;
       const int64_t m = (int64_t)a.n_bins + 1;
       const double* T = r.prefix;
       const double a0r = T[kcut] - T[k0], a0i = T[m + kcut] - T[m + k0];
-      const double ofs = to_double(k0) * a.df;
+      const double ofs = (double)k0 * a.df;
       const double a1r = (T[2 * m + kcut] - T[2 * m + k0]) - ofs * a0r;
       const double a1i = (T[3 * m + kcut] - T[3 * m + k0]) - ofs * a0i;
-      zr64 += to_double(rho_n.x) * a0r - to_double(rho_n.y) * a0i + sr1 * a1r - si1 * a1i;
-      zi64 += to_double(rho_n.x) * a0i + to_double(rho_n.y) * a0r + sr1 * a1i + si1 * a1r;
+      zr64 += (double)rho_n.x * a0r - (double)rho_n.y * a0i + sr1 * a1r - si1 * a1i;
+      zi64 += (double)rho_n.x * a0i + (double)rho_n.y * a0r + sr1 * a1i + si1 * a1r;
     }
     const double amp = sm.amp[si];
     Z = amp * hypot(zr64, zi64);

@@ -4,7 +4,7 @@ Workload (N = 1): the aligned-spin BNS population -- H1+L1, 20-1024 Hz at 1/128 
 (128,513 bins, complex64 data, FP64 PSD), coloured Gaussian noise, SNR 10-30; per event
 2^20 proposal samples over (Mc, q, chi1, chi2, t_c) from a Gaussian in the Fisher metric
 at the trigger; phase and distance marginalised.  One step = one event's batch:
-draw (Philox) -> fused waveform/projection/inner-product/marginalisation -> two-pass
+draw (Philox) -> fused waveform/projection/inner-product/marginalisation ->
 weight reduction.  Steps cycle over resident events; an L2 flush (256 MB write) runs
 between steps inside the timed region.
 
@@ -216,7 +216,9 @@ def run_gpu(args, rank, world):
     theta = torch.empty((P, n), dtype=torch.float64, device="cuda")
     lq, lp, ll = (torch.empty(n, dtype=torch.float64, device="cuda") for _ in range(3))
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
-    launches_per_step = 4  # draw, fused likelihood, reduce max, reduce sums
+    # draw, fused likelihood, reduction (not counted: the sample order's launches, which an
+    # event takes when its prior box reaches cuts inside the grid)
+    launches_per_step = 3
     like_events = []
 
     def step(i, timed):

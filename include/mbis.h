@@ -121,7 +121,8 @@ mbis_status mbis_set_metric(mbis_ctx* ctx, int32_t P, const int32_t* param_ids, 
 
 /* Draw n proposal samples (g of Eq. 5) with Philox4x32-10: sample i uses counter
  * (lo32(ctr0+i), hi32(ctr0+i), 2, block) and key (lo32(seed), hi32(seed)); Box-Muller
- * normals z, theta = mean + scale L z, RA and phi_c wrapped into [0, 2 pi), psi into
+ * normals z (in FP64 for MBIS_MIXED contexts, in 64-bit fixed point for MBIS_FP64 ones: the same
+ * to a few 1e-15), theta = mean + scale L z, RA and phi_c wrapped into [0, 2 pi), psi into
  * [0, pi).  Outputs (device): theta [P][n] SoA, log_q [n] = unwrapped Gaussian log
  * density, log_prior [n] (-inf outside the prior).  log_q / log_prior may be NULL.
  * Errors: MBIS_E_STATE (no metric), MBIS_E_INVALID (n < 0, null theta), MBIS_E_CUDA. */
@@ -140,9 +141,9 @@ mbis_status mbis_draw(mbis_ctx* ctx, uint64_t seed, uint64_t ctr0, int64_t n, do
  * Errors: MBIS_E_STATE, MBIS_E_INVALID, MBIS_E_UNSUPPORTED, MBIS_E_OOM, MBIS_E_CUDA. */
 mbis_status mbis_loglike(mbis_ctx* ctx, int64_t n, const double* theta, double* loglike, void* cuda_stream);
 
-/* Importance weights and Kish ESS (Eqs. 5-6), evidence Z = mean(w).  Two passes on the
- * device: m = max(log L + log pi - log g), then FP64 sums S1 = sum e^(log w - m),
- * S2 = sum e^(2 (log w - m)).  Inputs (device, n each).  weights_out (device, n) gets the
+/* Importance weights and Kish ESS (Eqs. 5-6), evidence Z = mean(w):
+ * m = max(log L + log pi - log g), then FP64 sums S1 = sum e^(log w - m),
+ * S2 = sum e^(2 (log w - m)), in one pass on the device (sums about each CTA's own maximum).  Inputs (device, n each).  weights_out (device, n) gets the
  * normalised weights e^(log w - m) / S1 when not NULL.  accumulate != 0 merges this batch
  * into the context's running state and reports the merged summary; 0 reports this batch
  * alone and leaves the running state untouched.  *out (host) receives the summary;

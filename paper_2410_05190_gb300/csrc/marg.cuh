@@ -23,8 +23,8 @@ constexpr int kGL48 = 48, kGL8 = 8;
 // the window's is left out
 constexpr float kDistSkip = 45.0f;
 constexpr int kGLSize = 2 * kGL48 + 2 * kGL8;
-// The rule without a peak: 24 panels of 8 points over the whole distance range, whose nodes do
-// not depend on the sample.  The FP32 node table goes on with their offsets d from the
+// The rule without a peak inside: 24 panels of 8 points over the whole distance range, whose nodes
+// do not depend on the sample.  The FP32 node table goes on with their offsets d from the
 // large-distance end and with expm1(d).
 constexpr int kDistFull = 24 * kGL8;
 constexpr int kGLTableF = kGLSize + 2 * kDistFull;  // floats of the FP32 table
@@ -222,6 +222,10 @@ __device__ __forceinline__ DistWindow dist_window(double Z, double H, const Dist
     d.whi = fminf(dc.span, rc + 12.0f * sig);
     d.window = d.wlo < d.whi;
     d.r_ref = fminf(fmaxf(rc, 0.0f), dc.span);
+    if (!d.window) {  // the peak lies beyond an end: the whole range about that end
+      d.wlo = 0.0f;
+      d.whi = dc.span;
+    }
   }
   d.u_ref = dc.u_lo * __expf(d.r_ref);
   d.phi_ref = log_i0_minus_x_f(d.Z * d.u_ref);
@@ -230,12 +234,14 @@ __device__ __forceinline__ DistWindow dist_window(double Z, double H, const Dist
   return d;
 }
 
-// The main rule: 48 nodes over the window, or the whole range's without one (the reference
-// point is then the large-distance end, so d.lo = 0 and d.hi = span).  node i: its offset and
-// expm1 of it.
+// The main rule: 48 nodes over the window, or the whole range's without one.  node i: its offset
+// and expm1 of it.  The whole range's are tabled for the reference point at the large-distance
+// end, lo = 0; a peak beyond the near end puts the reference there (the growing terms then vanish
+// where the integrand is largest), and its nodes are evaluated.
 __device__ __forceinline__ float2 dist_main_node(bool window, float lo, float hi, const float* gl, int i) {
-  if (!window) return make_float2(__ldg(gl + kGLSize + i), __ldg(gl + kGLSize + kDistFull + i));
-  const float d = dist_node_at(lo, hi, 1, 0, __ldg(gl + i));
+  if (!window && lo == 0.0f) return make_float2(__ldg(gl + kGLSize + i), __ldg(gl + kGLSize + kDistFull + i));
+  const float d = window ? dist_node_at(lo, hi, 1, 0, __ldg(gl + i))
+                         : dist_node_at(lo, hi, 24, i / kGL8, __ldg(gl + 2 * kGL48 + i % kGL8));
   return make_float2(d, expm1f(d));
 }
 __device__ __forceinline__ float dist_main_weight(bool window, float lo, float hi, const float* gl, int i) {

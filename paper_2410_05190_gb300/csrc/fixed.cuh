@@ -108,6 +108,16 @@ MBIS_HD int64_t mul32(Pair32 a, Pair32 b, int64_t c) {
   return add_high(madw(a.l, b.h, mulw(a.h, b.l)), madw(a.h, b.h, c));
 }
 
+// (ar, ai) += (wr + i wi) (co - i si), every factor in halves: with w in unit 2^-58 and the
+// sine and cosine in unit 2^-62 the sums have unit 2^-56.  The subtracted products negate high
+// halves only: a low half of -2^31 has no negative in 32 bits.
+MBIS_HD void add_rotated(Pair32 wr, Pair32 wi, Pair32 co, Pair32 si, int64_t& ar, int64_t& ai) {
+  const int64_t mr = madw(wi.h, si.l, madw(wi.l, si.h, madw(wr.h, co.l, mulw(wr.l, co.h))));
+  const int64_t mi = madw(-wr.h, si.l, madw(wr.l, -si.h, madw(wi.h, co.l, mulw(wi.l, co.h))));
+  ar = add_high(mr, madw(wi.h, si.h, madw(wr.h, co.h, ar)));
+  ai = add_high(mi, madw(wr.h, -si.h, madw(wi.h, co.h, ai)));
+}
+
 // ---- sine and cosine of a phase in turns ------------------------------------------------
 // The phase P counts 2^-64 turns.  Its nearest multiple of 1/128 turn is i / 128 + q / 4
 // (i = 0..31, a table entry; q the quadrant), the rest r 2^-64 turns with |r| <= 2^56.  With

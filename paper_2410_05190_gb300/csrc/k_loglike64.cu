@@ -462,13 +462,7 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
           trig_eval(cell, tc, ts, co64, si64);
           const Pair32 co = pair32(co64), si = pair32(si64);
           const int4 w = row[kPhaseInts / 4 + d];  // re (h, l), im (h, l)
-          if (k < kcut) {
-            // w e^(-i phi): (re co + im si, im co - re si)
-            const int64_t mr = madw(w.z, si.l, madw(w.w, si.h, madw(w.x, co.l, mulw(w.y, co.h))));
-            const int64_t mi = madw(-w.x, si.l, madw(-w.y, si.h, madw(w.z, co.l, mulw(w.w, co.h))));
-            ar[d] = add_high(mr, madw(w.z, si.h, madw(w.x, co.h, ar[d])));
-            ai[d] = add_high(mi, madw(-w.x, si.h, madw(w.z, co.h, ai[d])));
-          }
+          if (k < kcut) add_rotated(Pair32{w.x, w.y}, Pair32{w.z, w.w}, co, si, ar[d], ai[d]);
         }
       }
       const double scale = __longlong_as_double((int64_t)(max(E, -900) - 56 + 1023) << 52);

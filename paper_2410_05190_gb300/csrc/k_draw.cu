@@ -48,7 +48,8 @@ struct DrawTables {
   __align__(16) longlong2 log[128];
 };
 
-// x modulo the period: the quotient's floor from FP32, exact after one step either way
+// x modulo the period, in [0, period): the quotient's floor from FP32, exact after one step either
+// way; a number nearer to an end than its rounding (the step then lands on the other) is 0
 __device__ __forceinline__ double wrap_period(double x, double period) {
   const float turns = __fdividef((float)x, (float)period);
   if (fabsf(turns) < 65536.0f) {
@@ -57,12 +58,13 @@ __device__ __forceinline__ double wrap_period(double x, double period) {
     if (order_key(y) < 0 || order_key(y) >= order_key(period)) {
       k += order_key(y) < 0 ? -1.0f : 1.0f;
       y = fma(-(double)k, period, x);
+      if (order_key(y) < 0 || order_key(y) >= order_key(period)) y = 0.0;
     }
     return y;
   }
   double y = x - period * floor(x / period);
-  if (y >= period) y -= period;
   if (y < 0.0) y += period;
+  if (y >= period) y -= period;
   return y;
 }
 

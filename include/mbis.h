@@ -122,8 +122,8 @@ mbis_status mbis_set_metric(mbis_ctx* ctx, int32_t P, const int32_t* param_ids, 
 /* Draw n proposal samples (g of Eq. 5) with Philox4x32-10: sample i uses counter
  * (lo32(ctr0+i), hi32(ctr0+i), 2, block) and key (lo32(seed), hi32(seed)); Box-Muller
  * normals z (in FP64 for MBIS_MIXED contexts, in 64-bit fixed point for MBIS_FP64 ones: the same
- * to a few 1e-15), theta = mean + scale L z, RA and phi_c wrapped into [0, 2 pi), psi into
- * [0, pi).  Outputs (device): theta [P][n] SoA, log_q [n] = unwrapped Gaussian log
+ * to a few 1e-15, the log prior to an ulp of each of its terms), theta = mean + scale L z, RA and
+ * phi_c wrapped into [0, 2 pi), psi into [0, pi).  Outputs (device): theta [P][n] SoA, log_q [n] = unwrapped Gaussian log
  * density, log_prior [n] (-inf outside the prior).  log_q / log_prior may be NULL.
  * Errors: MBIS_E_STATE (no metric), MBIS_E_INVALID (n < 0, null theta), MBIS_E_CUDA. */
 mbis_status mbis_draw(mbis_ctx* ctx, uint64_t seed, uint64_t ctr0, int64_t n, double* theta, double* log_q,

@@ -275,8 +275,10 @@ MBIS_HD uint64_t uniform_mantissa(uint32_t a, int32_t& e) {
   return w << lz;
 }
 
-// ln x of a positive normal x = m 2^-63 2^e, unit 2^-52, from log_frac(m)
-MBIS_HD int64_t log_sum(int32_t e, int64_t frac) { return (int64_t)e * kLn2_52 + ((frac + e * kLn2_62 + 512) >> 10); }
+// ln x of a positive normal x = m 2^-63 2^e, unit 2^-53, from log_frac(m)
+MBIS_HD int64_t log_sum(int32_t e, int64_t frac) {
+  return (int64_t)e * (2 * kLn2_52) + ((frac + e * kLn2_62 + 256) >> 9);
+}
 struct LogArg {
   uint64_t m;
   int32_t e;
@@ -284,6 +286,21 @@ struct LogArg {
 MBIS_HD LogArg log_arg(double x) {
   const uint64_t b = double_bits(x);
   return LogArg{((b & 0xfffffffffffffull) | 0x10000000000000ull) << 11, (int32_t)((b >> 52) & 0x7ff) - 1023};
+}
+
+// ln(sin d / d) of 0 <= d < 1/8, unit 2^-62: with t = 64 d^2 the series
+// -t (1/384 + t (1/737280 + t (1/743178240 + ...))), whose next term is below 2^-58.
+MBIS_HD int64_t log_sinc(double d) {
+  constexpr double kUnit = 1152921504606846976.0;  // 2^60
+  const Pair28 D = pair28(to_fixed(d, 59));        // 8 d, unit 2^-56
+  const int64_t T = mul28(D, D, 0);
+  const uint32_t t = (uint32_t)(T >> 24);
+  const Pair28 tp = pair28(T);
+  uint32_t b = (uint32_t)(kUnit / (37800.0 * 16777216.0)) + mulhi_u(t, (uint32_t)(kUnit / (467775.0 * 1073741824.0)));
+  b = (uint32_t)(kUnit / (2835.0 * 262144.0)) + mulhi_u(t, b);
+  const int64_t c = (int64_t)(kUnit / (180.0 * 4096.0)) + mulhi_u(t, b);
+  const int64_t g = (int64_t)(kUnit / (6.0 * 64.0)) + mul28(tp, pair28(c), 0);
+  return -(mul28(tp, pair28(g), 0) * 4);
 }
 
 // ---- exponential ---------------------------------------------------------------------------

@@ -12,8 +12,8 @@
 // integer pipe, and the normals come in two arithmetics:
 //   * contexts of MBIS_FP64: fixed point throughout -- the Box-Muller logarithm, root, sine and
 //     cosine and the Cholesky sums (a normal's error is 2.8e-17 rms and 1.2e-15 at most over
-//     3 10^6 draws, against 2.4e-16 and 2.9e-15 in FP64) -- which leaves FP64 a conversion and
-//     a multiply-add per slot;
+//     3 10^6 draws, against 2.4e-16 and 2.9e-15 in FP64; a logarithm of the prior is within an ulp
+//     up to the poles) -- which leaves FP64 a conversion and a multiply-add per slot;
 //   * contexts of MBIS_MIXED: the library's FP64 functions for normals, density and prior, whose
 //     last bits these samples have always had.  The mixed likelihoods round in FP32, so a sample
 //     one FP64 ulp away can round to another log L (by up to 6e-8 of its spread, seen in 2 of 50
@@ -34,6 +34,8 @@ namespace mbis {
 namespace {
 
 constexpr int kDrawThreads = 128;
+constexpr double kPolar = 0.12;                    // rad (log_sinc holds below 1/8)
+constexpr double kPiTail = 1.2246467991473532e-16;  // pi less its nearest FP64 number
 
 struct DrawConsts {
   double lp_const;          // the prior's log-normalisation, all slots
@@ -162,8 +164,8 @@ __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawCons
     }
   }
   double mc = 0.0, q = 0.0;
-  bool inside = true;
-  int64_t log_sum50 = 0;  // the prior's logarithms, unit 2^-50
+  bool inside = true, polar = false;
+  int64_t log_sum51 = 0, polar53 = 0;  // the prior's logarithms, units 2^-51 and 2^-53
 #pragma unroll
   for (int p = 0; p < P; ++p) {
     double x = a.mean[p];
@@ -203,14 +205,27 @@ __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawCons
       continue;
     }
     if (id == kDec || id == kIota) {
-      int64_t co, si;
-      trig_of(tb, angle_turns(inside ? x : 1.0), co, si);
-      int64_t v = id == kDec ? co : si;
-      if (v < 1) v = 1;  // the ends of the range
-      const int lz = clz64((uint64_t)v);
-      log_sum50 += log_sum(1 - lz, log_mantissa(tb, (uint64_t)v << lz)) >> 2;
+      // ln cos(dec), ln sin(iota).  A sine in unit 2^-62 loses its relative accuracy towards the
+      // poles: within kPolar of one, ln d + ln(sin d / d) of the angle d from it
+      const double y = !inside ? 1.0 : id == kDec ? fabs(x) : x, pole = id == kDec ? 0.5 * kPi : kPi;
+      const bool face_on = id == kIota && order_key(y) < order_key(kPolar);
+      int64_t v;
+      if (face_on || order_key(y) > order_key(pole - kPolar)) {
+        const double d = face_on ? y : (pole - y) + (id == kDec ? 0.5 * kPiTail : kPiTail);
+        const LogArg arg = log_arg(d);
+        v = log_sum(arg.e, log_mantissa(tb, arg.m) + log_sinc(d));
+        if (order_key(d) == 0) inside = false;  // at the pole: ln 0
+      } else {
+        int64_t co, si;
+        trig_of(tb, angle_turns(y), co, si);
+        const uint64_t w = (uint64_t)(id == kDec ? co : si);
+        const int lz = clz64(w);
+        v = log_sum(1 - lz, log_mantissa(tb, w << lz));
+      }
+      polar53 += v;
+      polar = true;
     }
-    if (id == kDl) log_sum50 += log_of(tb, inside ? x : 1.0) >> 1;
+    if (id == kDl) log_sum51 += (log_of(tb, inside ? x : 1.0) + 1) >> 1;
   }
   // |d(m1, m2)/d(Mc, q)| = Mc (1 + q)^(2/5) q^(-6/5)
   if constexpr (!kFixed) {
@@ -222,10 +237,13 @@ __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawCons
   }
   if ((a.flags & MBIS_PRIOR_M1M2) && inside) {
     const int64_t lq = log_of(tb, q);
-    log_sum50 += (log_of(tb, mc) + __mul64hi(log_of(tb, 1.0 + q), 0x6666666666666666ll) - lq -
-                  __mul64hi(lq, 0x3333333333333333ll)) >> 2;
+    log_sum51 += (log_of(tb, mc) + __mul64hi(log_of(tb, 1.0 + q), 0x6666666666666666ll) - lq -
+                  __mul64hi(lq, 0x3333333333333333ll) + 2) >> 2;
   }
-  if (a.logp) a.logp[i] = inside ? fma((double)log_sum50, 0x1p-50, k.lp_const) : -INFINITY;
+  if (a.logp) {
+    if (polar) lp = fma((double)polar53, 0x1p-53, k.lp_const);
+    a.logp[i] = inside ? fma((double)log_sum51, 0x1p-51, polar ? lp : k.lp_const) : -INFINITY;
+  }
   if (a.logq) a.logq[i] = a.log_q_const - half_zz;
 }
 

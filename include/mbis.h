@@ -133,11 +133,16 @@ mbis_status mbis_draw(mbis_ctx* ctx, uint64_t seed, uint64_t ctr0, int64_t n, do
  * marginalised as the options say: PHASE -> ln I0(|Z|) - H/2; PHASE|DISTANCE ->
  * ln int p(d) I0(|Z1|/d) e^(-H1/(2 d^2)) dd; TIME -> ln mean_j e^(Re z_j - H/2).  theta
  * (device, [P][n] SoA as written by mbis_draw), loglike (device, n).  Samples with an
- * unphysical parameter (Mc <= 0, q <= 0, |chi| >= 1, d_L <= 0) get -inf.  A call with fewer
- * samples than fill the GPU shares each sample's bins among several CTAs through scratch the
- * context owns (allocated on first need, from its pool in the server), with results equal bit
- * for bit to an unsplit launch; calls on one context are therefore ordered on one stream (or
- * synchronised), like its reductions.
+ * unphysical parameter (Mc <= 0, q <= 0, |chi| >= 1, d_L <= 0) get -inf.  A MBIS_MIXED call with
+ * fewer samples than fill the GPU (136,192 on 152 SMs) on more than 8192 bins shares each
+ * sample's bins among several CTAs through scratch the context owns (16 bytes per sample and
+ * 8192 bins, allocated on first need, from its pool in the server, and kept), with results equal
+ * bit for bit to an unsplit launch; calls on one context are therefore ordered on one stream (or
+ * synchronised), like its reductions.  Calls of up to four times as many samples do so through a
+ * second scratch, which the context keeps in order itself over streams and threads and does
+ * without (in whole tiles, the same bits) under stream capture or when memory is short.  In
+ * MBIS_FP64 the order of a sample's sums follows the size of the call: the last bits of its log L
+ * are those of any other call of as many samples.
  * Errors: MBIS_E_STATE, MBIS_E_INVALID, MBIS_E_UNSUPPORTED, MBIS_E_OOM, MBIS_E_CUDA. */
 mbis_status mbis_loglike(mbis_ctx* ctx, int64_t n, const double* theta, double* loglike, void* cuda_stream);
 

@@ -49,17 +49,51 @@ double q_integral(double a, double b) {
   return s;
 }
 
-// scratch of split folded launches of up to n samples
-cudaError_t split_scratch(mbis_ctx* c, int32_t parts, int64_t n) {
-  dfree(c, c->d_zpart);
-  dfree(c, c->d_amp);
-  dfree(c, c->d_kcut);
-  c->split_cap = 0;
-  cudaError_t e = dalloc(c, &c->d_zpart, sizeof(double2) * (size_t)parts * (size_t)n);
-  if (e == cudaSuccess) e = dalloc(c, &c->d_amp, sizeof(double) * (size_t)n);
-  if (e == cudaSuccess) e = dalloc(c, &c->d_kcut, sizeof(int32_t) * (size_t)n);
-  if (e == cudaSuccess) c->split_cap = n;
+void free_split(mbis_ctx* c, SplitScratch& sc) {
+  dfree(c, sc.zpart);
+  dfree(c, sc.amp);
+  dfree(c, sc.kcut);
+  sc.cap = 0;
+}
+
+// room for split folded launches of n samples; none is kept when not all can be had
+cudaError_t grow_split(mbis_ctx* c, SplitScratch& sc, int32_t parts, int64_t n) {
+  if (sc.cap >= n) return cudaSuccess;
+  free_split(c, sc);
+  cudaError_t e = dalloc(c, &sc.zpart, sizeof(double2) * (size_t)parts * (size_t)n);
+  if (e == cudaSuccess) e = dalloc(c, &sc.amp, sizeof(double) * (size_t)n);
+  if (e == cudaSuccess) e = dalloc(c, &sc.kcut, sizeof(int32_t) * (size_t)n);
+  if (e == cudaSuccess)
+    sc.cap = n;
+  else
+    free_split(c, sc);
   return e;
+}
+
+// The scratch of a split launch beyond one wave of tiles.  There it only buys speed, so such calls
+// stay as free as those of whole tiles, which need none: a lock, and an event that the next use
+// waits for, let them run on any stream and thread; under capture (the graph would outlive the
+// buffers) and when the memory cannot be had the call is refused the scratch and keeps whole
+// tiles.  Hold the lock until wide_done is recorded after the launch.
+std::unique_lock<std::mutex> wide_scratch(mbis_ctx* c, int32_t parts, int64_t n, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(s, &cap);
+  if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    std::unique_lock<std::mutex> lock(c->wide_mu);
+    // allocations do not end a capture that goes on in another thread
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!c->wide_done)
+      e = cudaEventCreateWithFlags(&c->wide_done, cudaEventDisableTiming);
+    else if (c->pool && c->wide.cap < n)
+      e = cudaStreamWaitEvent(c->stream, c->wide_done, 0);  // the old buffers are freed on this stream
+    if (e == cudaSuccess) e = grow_split(c, c->wide, parts, n);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->wide_done, 0);
+    if (e == cudaSuccess) return lock;
+  }
+  (void)cudaGetLastError();
+  return {};
 }
 
 void free_tables(mbis_ctx* c) {
@@ -650,12 +684,12 @@ void mbis_destroy(mbis_ctx* c) {
   if (!c) return;
   rb_free(c);
   free_tables(c);
-  dfree(c, c->d_zpart);
+  free_split(c, c->split);
+  free_split(c, c->wide);
+  if (c->wide_done) cudaEventDestroy(c->wide_done);
   dfree(c, c->d_tperm);
   dfree(c, c->d_thist);
   c->tperm_cap = 0;
-  dfree(c, c->d_amp);
-  dfree(c, c->d_kcut);
   dfree(c, c->d_strain);
   dfree(c, c->d_psd64);
   dfree(c, c->d_basis);
@@ -769,29 +803,31 @@ mbis_status mbis_loglike(mbis_ctx* c, int64_t n, const double* theta, double* lo
     // GPU stays full to the end, at the price of a repeated set-up (~0.1 of a part's time) and
     // of the epilogue.  Measured on 16-part grids (ms, whole tiles -> one-part pieces):
     // 10^4 samples 0.90, 2^17 7.9 (both always split); 2*10^5 13.0 -> 11.9, 2^18 16.3 -> 15.5,
-    // 4*10^5 24.0 -> 23.5; two-part pieces lose (2^16: 4.18 against 4.10).
+    // 4*10^5 24.0 -> 23.5; two-part pieces lose (2^16: 4.18 against 4.10).  The sums of the parts
+    // take 16 bytes per sample and part, in scratch that the context keeps; the same bits either
+    // way.
     LikeArgs b = a;
     const int64_t tiles = (n + kMixedThreads - 1) / kMixedThreads, slots = (int64_t)c->n_sms * kFoldCtasPerSm;
     const int32_t parts = (c->n_bins + kPartBins - 1) / kPartBins;
-    b.split = parts > 1 && tiles < 4 * slots ? parts : 1;
-    if (b.split > 1 && tiles >= slots && c->split_cap < n) {
-      // beyond one wave the scratch (16 bytes per sample and part) only buys speed: whole tiles
-      // when it cannot be had, or while the stream is being captured
-      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-      CU_TRY(c, cudaStreamIsCapturing(s, &cap));
-      if (cap != cudaStreamCaptureStatusNone || split_scratch(c, parts, n) != cudaSuccess) {
-        (void)cudaGetLastError();
-        b.split = 1;
-      }
-    }
     if (const mbis_status r = sample_order(c, a, kFoldOrderGran, s, &b.perm); r != MBIS_OK) return r;
-    if (b.split > 1) {
-      if (c->split_cap < n) CU_TRY(c, split_scratch(c, parts, n));
-      b.zpart = c->d_zpart;
-      b.amp_out = c->d_amp;
-      b.kcut_out = c->d_kcut;
+    std::unique_lock<std::mutex> wide;
+    const SplitScratch* sc = nullptr;
+    if (parts > 1 && tiles < slots) {
+      CU_TRY(c, grow_split(c, c->split, parts, n));
+      sc = &c->split;
+    } else if (parts > 1 && tiles < 4 * slots) {
+      wide = wide_scratch(c, parts, n, s);
+      if (wide.owns_lock()) sc = &c->wide;
     }
-    CU_TRY(c, launch_loglike_mixed(b, s));
+    b.split = sc ? parts : 1;
+    if (sc) {
+      b.zpart = sc->zpart;
+      b.amp_out = sc->amp;
+      b.kcut_out = sc->kcut;
+    }
+    const cudaError_t le = launch_loglike_mixed(b, s);
+    if (wide.owns_lock()) CU_TRY(c, cudaEventRecord(c->wide_done, s));
+    CU_TRY(c, le);
   }
   return MBIS_OK;
 }

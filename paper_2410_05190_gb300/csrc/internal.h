@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -270,6 +271,14 @@ DrawArgs make_draw_args(const mbis_ctx* c, uint64_t seed, uint64_t ctr0, int64_t
 LikeArgs make_like_args(const mbis_ctx* c, int64_t n, const double* theta, double* loglike);
 mbis_status sample_order(mbis_ctx* c, const LikeArgs& a, int32_t gran, cudaStream_t s, const int32_t** perm);
 void rb_free(mbis_ctx* c);
+
+// Scratch of split folded launches: the sums of the parts, each sample's amplitude and cut.
+struct SplitScratch {
+  double2* zpart = nullptr;
+  double* amp = nullptr;
+  int32_t* kcut = nullptr;
+  int64_t cap = 0;  // samples it holds
+};
 }  // namespace mbis
 
 // the context behind the opaque handle
@@ -303,11 +312,11 @@ struct mbis_ctx {
   uint64_t gen = 0;          // bumped whenever the tables or the proposal change (batches re-capture)
   uint64_t tables_gen = 0;   // bumped whenever the tables are rebuilt (mbis_set_metric)
   int32_t n_sms = 0;         // SMs of the context's device
-  // scratch of split folded launches (grown on demand)
-  double2* d_zpart = nullptr;
-  double* d_amp = nullptr;
-  int32_t* d_kcut = nullptr;
-  int64_t split_cap = 0;     // samples x parts the scratch holds
+  // scratch of split folded launches (grown on demand): of calls that do not fill the GPU, which
+  // the caller keeps in order, and of larger ones, which the context does (capi.cu)
+  mbis::SplitScratch split, wide;
+  std::mutex wide_mu;
+  cudaEvent_t wide_done = nullptr;  // the last use of `wide`
   // scratch of a launch's sample order (grown on demand)
   int32_t* d_tperm = nullptr;
   int32_t* d_thist = nullptr;

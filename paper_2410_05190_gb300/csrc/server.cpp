@@ -95,9 +95,12 @@ int64_t request_footprint(const Request& q) {
   size_t t = ctx_footprint_bytes(r.event.n_det, r.grid.n_bins, r.event.dtype, r.opts, is_fold(q.ids));
   t += round_alloc(sizeof(double) * (size_t)r.ess.batch * r.P) + 4 * round_alloc(sizeof(double) * (size_t)r.ess.batch);
   if (r.opts.precision == MBIS_MIXED && !(r.opts.marg & MBIS_MARG_TIME) && is_fold(q.ids)) {
-    // scratch of a split folded launch: per-part sums, amplitude and cut per sample
+    // scratch of split folded launches (per-part sums, amplitude and cut per sample): of those
+    // below a wave of tiles, and of those of one to four
     const size_t parts = ((size_t)r.grid.n_bins + kPartBins - 1) / kPartBins, nb = (size_t)r.ess.batch;
-    t += round_alloc(16 * parts * nb) + round_alloc(8 * nb) + round_alloc(4 * nb);
+    const size_t wave = (size_t)152 * kFoldCtasPerSm * kMixedThreads;
+    for (const size_t n : {std::min(nb, wave), nb > wave - kMixedThreads ? std::min(nb, 4 * wave) : 0})
+      t += round_alloc(16 * parts * n) + round_alloc(8 * n) + round_alloc(4 * n);
   }
   if (r.opts.precision == MBIS_MIXED) {
     // sample order of a launch: the permutation and the key counts

@@ -5,8 +5,9 @@
 // One launch reads the inputs once.  Each CTA takes the maximum m_b of its own samples, sums
 // e^(lw - m_b) and its square, and leaves (m_b, S1_b, S2_b); the last CTA to finish (atomic
 // ticket) folds the partials about m = max m_b in a fixed order with all its threads, so the
-// result does not depend on scheduling.  When weights are asked for, the first launch leaves
-// e^(lw - m_b) in them and a second one scales each CTA's samples by e^(m_b - m) / S1.
+// result does not depend on scheduling.  When weights are asked for, the first launch leaves lw
+// in them and a second one makes e^(lw - m) / S1 of it: e^(lw - m_b) scaled by e^(m_b - m) / S1
+// would save the second exponential and carry the rounding of a further one.
 // The FP64 pipe (64 clocks per warp instruction and SM quarter) bounds the pass and not HBM:
 // the exponentials run in fixed point (fixed.cuh: 0.76 ulp at most, 0.31 rms, where FP64 took
 // some 30 instructions), the maxima on the integer pipe, and a warp's two sums fold with five
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(int64_t n, const
     const double e = shifted_exp(lw, m);
     s1 += e;
     s2 = fma(e, e, s2);
-    if (w) w[i] = e;
+    if (w) w[i] = lw;
   };
 #pragma unroll
   for (int r = 0; r < kKeep; ++r) {
@@ -165,20 +166,15 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(int64_t n, const
   }
 }
 
-// the same grid as reduce_kernel: this CTA's samples are those its maximum belongs to
 __global__ void __launch_bounds__(kReduceThreads) weights_kernel(int64_t n, ReduceScratch scr, double* w) {
-  __shared__ double sh_f;
-  const double m = scr.result[0];
-  if (threadIdx.x == 0) {
-    const double mb = scr.partials[3 * blockIdx.x];
-    sh_f = (order_key(mb) == order_key(m) ? 1.0 : shifted_exp(mb, m)) / scr.result[1];
-  }
+  __shared__ double sh_inv;
+  if (threadIdx.x == 0) sh_inv = 1.0 / scr.result[1];
   __syncthreads();
-  const double f = sh_f;
-  const bool zero = order_key(m) <= kKeyMin;
+  const double m = scr.result[0], inv = sh_inv;
+  const bool any = order_key(m) > kKeyMin;
   const int64_t stride = (int64_t)gridDim.x * kReduceThreads;
   for (int64_t i = (int64_t)blockIdx.x * kReduceThreads + threadIdx.x; i < n; i += stride)
-    w[i] = zero ? 0.0 : w[i] * f;
+    w[i] = any ? shifted_exp(w[i], m) * inv : 0.0;
 }
 
 // ---- the ordered form, for the refits of the ESS loop

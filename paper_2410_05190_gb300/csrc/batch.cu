@@ -21,6 +21,50 @@
 
 using namespace mbis;
 
+namespace {
+
+// The side streams of a capture: branches fork from the main stream and join it again.  Only the
+// graph's shape comes from them; the batch keeps them for its next capture (there is one in every
+// step after a moved proposal, and creating and destroying them takes some 30 of its 200 us).
+struct Branches {
+  static constexpr int kMax = 8;
+  cudaStream_t s[kMax] = {};
+  cudaEvent_t fork = nullptr, join[kMax] = {};
+  int n = 0;
+  // makes what is missing of `want` branches
+  cudaError_t init(int want) {
+    cudaError_t e = fork ? cudaSuccess : cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    while (e == cudaSuccess && n < want && n < kMax) {
+      if (!s[n]) e = cudaStreamCreateWithFlags(&s[n], cudaStreamNonBlocking);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[n], cudaEventDisableTiming);
+      if (e == cudaSuccess) ++n;
+    }
+    return e;
+  }
+  cudaError_t open(cudaStream_t main) {
+    cudaError_t e = cudaEventRecord(fork, main);
+    for (int i = 0; e == cudaSuccess && i < n; ++i) e = cudaStreamWaitEvent(s[i], fork, 0);
+    return e;
+  }
+  cudaError_t close(cudaStream_t main) {
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; e == cudaSuccess && i < n; ++i) {
+      e = cudaEventRecord(join[i], s[i]);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(main, join[i], 0);
+    }
+    return e;
+  }
+  ~Branches() {
+    if (fork) cudaEventDestroy(fork);
+    for (int i = 0; i < kMax; ++i) {
+      if (join[i]) cudaEventDestroy(join[i]);
+      if (s[i]) cudaStreamDestroy(s[i]);
+    }
+  }
+};
+
+}  // namespace
+
 struct mbis_batch {
   int32_t n = 0;
   std::vector<mbis_ctx*> ctx;
@@ -45,6 +89,7 @@ struct mbis_batch {
   cudaStream_t stream = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;
+  Branches branches;
 };
 
 namespace {
@@ -111,50 +156,14 @@ LikeArgs batch_args(const mbis_batch* b, int i) {
   return a;
 }
 
-// The side streams of one capture: branches fork from the main stream and join it again.
-// Only the graph's shape comes from them, so they live as long as the capture.
-struct Branches {
-  static constexpr int kMax = 8;
-  cudaStream_t s[kMax] = {};
-  cudaEvent_t fork = nullptr, join[kMax] = {};
-  int n = 0;
-  cudaError_t init(int want) {
-    cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
-    for (; e == cudaSuccess && n < want && n < kMax; ++n) {
-      e = cudaStreamCreateWithFlags(&s[n], cudaStreamNonBlocking);
-      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[n], cudaEventDisableTiming);
-    }
-    return e;
-  }
-  cudaError_t open(cudaStream_t main) {
-    cudaError_t e = cudaEventRecord(fork, main);
-    for (int i = 0; e == cudaSuccess && i < n; ++i) e = cudaStreamWaitEvent(s[i], fork, 0);
-    return e;
-  }
-  cudaError_t close(cudaStream_t main) {
-    cudaError_t e = cudaSuccess;
-    for (int i = 0; e == cudaSuccess && i < n; ++i) {
-      e = cudaEventRecord(join[i], s[i]);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(main, join[i], 0);
-    }
-    return e;
-  }
-  ~Branches() {
-    if (fork) cudaEventDestroy(fork);
-    for (int i = 0; i < kMax; ++i) {
-      if (join[i]) cudaEventDestroy(join[i]);
-      if (s[i]) cudaStreamDestroy(s[i]);
-    }
-  }
-};
-
 // Enqueue one step on b->stream, under capture.  The events' draws and orders depend on the
 // counters alone, and their reductions on the likelihoods alone, so they run on branches side
 // by side: a draw or a reduction of 2^14 .. 2^17 samples is a chain of FP64 latencies on part
 // of the GPU (a step of 8 events of such sizes takes 12.25 ms with them one after another,
 // 12.01 ms on branches).  Events that share a context share its reduction scratch and so a
 // branch.
-mbis_status enqueue_step(mbis_batch* b, Branches& br) {
+mbis_status enqueue_step(mbis_batch* b) {
+  Branches& br = b->branches;
   std::vector<cudaStream_t> on(b->n);
   std::unordered_map<const mbis_ctx*, cudaStream_t> taken;
   for (int i = 0; i < b->n; ++i) on[i] = taken.emplace(b->ctx[i], br.s[i % br.n]).first->second;
@@ -182,10 +191,9 @@ mbis_status capture(mbis_batch* b) {
   if (b->graph) cudaGraphDestroy(b->graph);
   b->exec = nullptr;
   b->graph = nullptr;
-  Branches br;
-  B_TRY(br.init(std::min(b->n, Branches::kMax)));
+  B_TRY(b->branches.init(b->n));
   B_TRY(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-  const mbis_status st = enqueue_step(b, br);
+  const mbis_status st = enqueue_step(b);
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(b->stream, &g);
   if (st != MBIS_OK) {

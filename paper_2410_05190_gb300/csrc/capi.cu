@@ -442,11 +442,14 @@ mbis_status mbis::create_ctx(const mbis_event* ev, const double* psd, const mbis
     float glf[kGLSize];
     fill_gauss_legendre(gl);
     fill_gauss_legendre_f32(glf);
-    CREATE_TRY(dalloc(c, &c->d_gl, sizeof(gl) + sizeof(float) * kGLTableF));
+    // the whole range's nodes where they are read: with the distance marginalised
+    const bool dist = mg & MBIS_MARG_DISTANCE;
+    CREATE_TRY(dalloc(c, &c->d_gl, sizeof(gl) + sizeof(float) * (dist ? kGLTableF : kGLSize)));
     CREATE_TRY(cudaMemcpyAsync(c->d_gl, gl, sizeof(gl), cudaMemcpyHostToDevice, s));
     CREATE_TRY(cudaMemcpyAsync(c->d_gl + kGLSize, glf, sizeof(glf), cudaMemcpyHostToDevice, s));
-    CREATE_TRY(launch_dist_nodes(dist_const(opts->dmin_mpc, opts->dmax_mpc).span,
-                                 reinterpret_cast<float*>(c->d_gl + kGLSize), s));
+    if (dist)
+      CREATE_TRY(launch_dist_nodes(dist_const(opts->dmin_mpc, opts->dmax_mpc).span,
+                                   reinterpret_cast<float*>(c->d_gl + kGLSize), s));
     CREATE_TRY(cudaStreamSynchronize(s));  // gl, glf are on this stack frame
   }
   CREATE_TRY(dalloc(c, &c->d_err, sizeof(int32_t)));
@@ -532,7 +535,8 @@ size_t mbis::ctx_footprint_bytes(int32_t n_det, int32_t n_bins, int32_t dtype, c
   const size_t n = (size_t)n_bins, nd = (size_t)n_det, nb = n * nd;
   size_t t = 0;
   t += round_alloc((dtype == MBIS_C128 ? 16 : 8) * nb) + round_alloc(8 * nb);  // strain, PSD
-  t += round_alloc(8 * kNumBasis * n) + round_alloc(8 * kGLSize + 4 * kGLTableF) + round_alloc(4);
+  t += round_alloc(8 * kNumBasis * n) + round_alloc(4) +
+       round_alloc(8 * kGLSize + 4 * (opts.marg & MBIS_MARG_DISTANCE ? kGLTableF : kGLSize));
   t += round_alloc(24 * kReduceBlocks) + round_alloc(4) + round_alloc(32);
   t += round_alloc(8 * (size_t)moments_partials_size(kMaxP)) + round_alloc(4) + round_alloc(8 * kMomentSums);
   const size_t rows = fold ? 1 : nd;

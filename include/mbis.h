@@ -630,6 +630,12 @@ mbis_status mbis_debug_ff_sincos(int64_t n, const double* x, double* sin_out, do
 mbis_status mbis_debug_setup_pair(int64_t n, const double* params, double f_lo, double df, int32_t n_bins,
                                   double* out, void* cuda_stream);
 
+/* Self-test of mbis_credible_levels' fallbacks (not in the paper): the same with clusters of at
+ * most max_ctas CTAs per slot -- 16, as it starts with, 8 or 1, as where the GPU cannot place
+ * larger ones.  Errors: as mbis_credible_levels. */
+mbis_status mbis_debug_credible_levels(int64_t n, int32_t P, const double* theta, const double* weights,
+                                       const double* ref, double* levels, int32_t max_ctas, void* cuda_stream);
+
 /* Library build/version string. */
 const char* mbis_version(void);
 

@@ -150,6 +150,7 @@ def _load():
         "mbis_debug_ff_sincos": [i64, p, p, p, p],
         "mbis_debug_setup_pair": [i64, p, d, d, i32, p, p],
         "mbis_credible_levels": [i64, i32, p, p, p, p, p],
+        "mbis_debug_credible_levels": [i64, i32, p, p, p, p, i32, p],
         "mbis_rb_setup": [p, p, i32, p],
         "mbis_rb_loglike": [p, i64, p, p, p],
         "mbis_rb_edges": [p, p, d, d, i32, p, p],
@@ -458,6 +459,13 @@ def mbis_debug_setup_pair(n, params, f_lo, df, n_bins, out, stream=None):
     """FP64 and float-float per-sample set-up side by side (a self-test; out [2][12][n])."""
     _check(_lib.mbis_debug_setup_pair(int(n), _dev(params), float(f_lo), float(df), int(n_bins), _dev(out),
                                       _stream(stream)))
+
+
+def mbis_debug_credible_levels(n, theta, weights, ref, levels, max_ctas, stream=None):
+    """mbis_credible_levels with clusters of at most max_ctas CTAs (a self-test)."""
+    r, pr = _host(ref, np.float64)
+    _check(_lib.mbis_debug_credible_levels(n, len(r), _dev(theta), _dev(weights), pr, _dev(levels), int(max_ctas),
+                                           _stream(stream)))
 
 
 NOALLOC_MAX_SAMPLES = 16777216

@@ -141,8 +141,8 @@ mbis_status mbis_draw(mbis_ctx* ctx, uint64_t seed, uint64_t ctr0, int64_t n, do
  * synchronised), like its reductions.  Calls of up to four times as many samples do so through a
  * second scratch, which the context keeps in order itself over streams and threads and does
  * without (in whole tiles, the same bits) under stream capture or when memory is short.  In
- * MBIS_FP64 the order of a sample's sums follows the size of the call: the last bits of its log L
- * are those of any other call of as many samples.
+ * MBIS_FP64 without TIME the order of a sample's sums follows the size of the call: the last bits
+ * of its log L are those of any other call of as many samples.
  * Errors: MBIS_E_STATE, MBIS_E_INVALID, MBIS_E_UNSUPPORTED, MBIS_E_OOM, MBIS_E_CUDA. */
 mbis_status mbis_loglike(mbis_ctx* ctx, int64_t n, const double* theta, double* loglike, void* cuda_stream);
 

@@ -18,10 +18,11 @@
 // CTAs shares a tile of 32 samples, its warps taking the chunks in turn, and folds the sums
 // through distributed shared memory in a fixed order, so the launch needs no scratch.  The
 // per-sample set-up is spread over the CTA's warps, and the distance integral's nodes over the
-// cluster's warps.  Phase terms beyond 2^40 turns and non-finite data fall back to FP64 per
-// bin.  Bound by the integer multiply-adds (86 per warp and bin, 4 clocks each).  Measured on a
-// GB300, 4096 samples: 52.4 ms before and 6.6 ms now on 128,513 bins with phase and distance
-// marginalised; 291 us and 56 us on 1969 bins (240 live) with the phase marginalised.
+// cluster's warps.  A sample with phase terms beyond 2^40 turns, and all samples on 32 bins with
+// data that are not finite, are summed in FP64 per bin.  Bound by the integer multiply-adds (86
+// per warp and bin, 4 clocks each).  Measured on a GB300, 4096 samples: 52.4 ms before and 6.6 ms
+// now on 128,513 bins with phase and distance marginalised; 291 us and 56 us on 1969 bins (240
+// live) with the phase marginalised.
 //
 // loglike_fp64_time_kernel (time marginalisation): one warp per sample, lanes over bins, every
 // bin in FP64; the per-bin integrand a_k = A sum_d P_d c_dk e^(-i phi_dk) of 32
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
 #pragma unroll
     for (int d = 0; d < ROWS; ++d) T = max(T, exponent_above(sm.resp[2][d][lane]) + g.eb[kNumBasis - 1]);
   }
-  const bool far = __any_sync(0xffffffffu, T > kMaxTurnsExp);  // warp-uniform, the same in every warp
+  const bool far = T > kMaxTurnsExp;  // this lane's bins in FP64; its neighbours' are not touched
   T = min(T, kMaxTurnsExp);
   Pair32 c[kNumBasis], cd[FOLD ? 1 : ROWS];
 #pragma unroll
@@ -368,6 +369,7 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
   }
   const int32_t shift = T + 8;  // to 2^-64 turns
   const int32_t kcut = sm.kcut[lane];
+  const int32_t kfix = far ? 0 : kcut;  // bins to sum in fixed point
   const int32_t kmax = __reduce_max_sync(0xffffffffu, kcut);
   const Pair32 trig_c = pair32(kTrigTable[lane][0]), trig_s = pair32(kTrigTable[lane][1]);
 
@@ -395,7 +397,7 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
 #pragma unroll
     for (int d = 0; d < ROWS; ++d) E = max(E, max(exponent_above(nw[d].x), exponent_above(nw[d].y)));
     E = __reduce_max_sync(0xffffffffu, E);
-    const bool slow = far || E > 900 || (E < -900 && E > -1022);
+    const bool slow = E > 900 || (E < -900 && E > -1022);  // the chunk's data: warp-uniform
     const int32_t k_end = min(k0 + g.chunk, kmax);
     if (!slow) {
       int32_t* row = sm.stage[warp][lane];
@@ -462,7 +464,7 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
           trig_eval(cell, tc, ts, co64, si64);
           const Pair32 co = pair32(co64), si = pair32(si64);
           const int4 w = row[kPhaseInts / 4 + d];  // re (h, l), im (h, l)
-          if (k < kcut) add_rotated(Pair32{w.x, w.y}, Pair32{w.z, w.w}, co, si, ar[d], ai[d]);
+          if (k < kfix) add_rotated(Pair32{w.x, w.y}, Pair32{w.z, w.w}, co, si, ar[d], ai[d]);
         }
       }
       const double scale = __longlong_as_double((int64_t)(max(E, -900) - 56 + 1023) << 52);
@@ -471,7 +473,8 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
         zr[d] = fma((double)ar[d], scale, zr[d]);
         zi[d] = fma((double)ai[d], scale, zi[d]);
       }
-    } else {
+    }
+    if (slow || far) {
 #pragma unroll 1
       for (int32_t k = k0; k < min(k_end, kcut); ++k) {
         double t = sm.C[kNumBasis][lane];

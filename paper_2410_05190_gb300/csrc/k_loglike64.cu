@@ -5,10 +5,12 @@
 // loglike_fp64_kernel (no, phase, or phase and distance marginalisation).  An FP64 instruction
 // holds a quarter of an SM for 64 clocks on the GB300, so a bin that evaluates its nine-term
 // phase, a sincospi and a complex multiply-add in FP64 (the version before) costs 3750 clocks
-// per warp.  Every one of these quantities is bounded, and 64-bit integers carry them further
-// than FP64 does (fixed.cuh): per bin and warp
+// per warp.  Every one of these quantities is bounded, and 64-bit integers carry them
+// (fixed.cuh): per bin and warp
 //   * the phase in turns modulo one, sum_j C_j B_j(f_k), 29 multiply-adds of 32-bit halves with
-//     a unit of 2^-56 of the sample's largest phase term (FP64 rounds each term at 2^-53);
+//     a unit of 2^-56 of the sample's largest phase term on the grid.  FP64 rounds each bin's own
+//     terms at 2^-53: coarser where they are largest, finer where they have fallen below an
+//     eighth of that;
 //   * its sine and cosine to 2.7e-17 (a table of 32 entries held one per lane, fetched by
 //     shuffles, and the Taylor series of the rest: 36 multiply-adds);
 //   * the multiply-add with the data, scaled by the largest value of 32 bins, into 64-bit sums
@@ -541,7 +543,7 @@ __global__ void __launch_bounds__(kThreads64, ROWS == 1 ? 3 : 2) loglike_fp64_ke
           ll = log_i0(modulus(X, Y)) - 0.5 * H;
         if (active) a.out[s] = valid ? ll : -INFINITY;
       } else {
-        // the window of log_distance_marginal, and which of the ranges beside it count: G has
+        // the peak's window (marg.cuh), and which of the ranges beside it count: G has
         // at most one maximum, so a range without it is largest at its ends; one whose ends
         // lie 50 below the window's peak adds less than e^-49 (FP64 resolves e^-36)
         const double Z = modulus(X, Y);
@@ -644,7 +646,6 @@ cudaError_t launch_fp64(const Fp64Args& g, int R, int64_t tiles, cudaStream_t s)
   auto kernel = loglike_fp64_kernel<ROWS, FOLD>;
   constexpr int kBytes = (int)sizeof(Smem64<ROWS>);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(tiles * R));

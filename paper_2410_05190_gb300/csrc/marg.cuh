@@ -9,9 +9,10 @@
 // has, for a loud match (Z1^2 > 14 H1), a peak at u = e^s solving H1 u^2 - Z1 u + 7/2 = 0
 // (large-argument I1/I0 ~ 1 - 1/(2x)) of width 1/sqrt(Z1 u - 7).  A 48-point Gauss-Legendre
 // rule covers +-12 widths about the peak and 8-point composite rules the rest of the
-// range; without a peak the whole range gets a 24-panel composite 8-point rule.  Sums run
-// as an online log-sum-exp: in FP64 in log_distance_marginal (the FP64 path), in FP32 about
-// an FP64 reference value in log_distance_marginal_mixed (the mixed-precision kernels).
+// range; without a peak inside it the whole range gets a 24-panel composite 8-point rule.  Sums
+// run as an online log-sum-exp: in FP64 in the double-precision kernel (k_loglike64.cu, which
+// shares the nodes among its warps), in FP32 about an FP64 reference value in
+// log_distance_marginal_mixed and its pieces (the mixed-precision kernels).
 #pragma once
 #include "physics.cuh"
 
@@ -51,49 +52,6 @@ struct LogSumExp {
   }
   __device__ __forceinline__ double value() const { return m + log(acc); }
 };
-
-__device__ __forceinline__ void dist_rule(LogSumExp& L, double a, double b, int panels, int n, const double* x,
-                                          const double* w, double Z, double H, double c0) {
-  const double h = (b - a) / panels;
-  for (int p = 0; p < panels; ++p) {
-    const double mid = a + (p + 0.5) * h, half = 0.5 * h;
-    for (int i = 0; i < n; ++i) {
-      const double s = mid + half * x[i];
-      const double u = exp(s);
-      const double g = c0 - 3.0 * s + log_i0(Z * u) - 0.5 * H * u * u;
-      L.add(g, half * w[i]);
-    }
-  }
-}
-
-__device__ __forceinline__ double log_distance_marginal(double Z, double H, double dmin, double dmax,
-                                                        const double* gl) {
-  const double* x48 = gl;
-  const double* w48 = gl + kGL48;
-  const double* x8 = gl + 2 * kGL48;
-  const double* w8 = gl + 2 * kGL48 + kGL8;
-  const double c0 = log(3.0 / (dmax * dmax * dmax - dmin * dmin * dmin));
-  const double s_lo = -log(dmax), s_hi = -log(dmin);
-  LogSumExp L;
-  bool window = false;
-  double wlo = s_lo, whi = s_hi;
-  if (H > 0.0 && Z * Z > 14.0 * H) {
-    const double u = (Z + sqrt(Z * Z - 14.0 * H)) / (2.0 * H);
-    const double sig = 1.0 / sqrt(fmax(Z * u - 7.0, 1e-300));
-    const double sc = log(u);
-    wlo = fmax(s_lo, sc - 12.0 * sig);
-    whi = fmin(s_hi, sc + 12.0 * sig);
-    window = wlo < whi;
-  }
-  if (window) {
-    dist_rule(L, wlo, whi, 1, kGL48, x48, w48, Z, H, c0);
-    if (wlo > s_lo) dist_rule(L, s_lo, wlo, 8, kGL8, x8, w8, Z, H, c0);
-    if (whi < s_hi) dist_rule(L, whi, s_hi, 8, kGL8, x8, w8, Z, H, c0);
-  } else {
-    dist_rule(L, s_lo, s_hi, 24, kGL8, x8, w8, Z, H, c0);
-  }
-  return L.value();
-}
 
 // ln I0(x) - x in FP32 (x >= 0), slowly varying, so FP32 keeps its absolute accuracy.  The
 // polynomial approximations of Abramowitz & Stegun 9.8.1 (x < 3.75: I0 in (x/3.75)^2) and
@@ -190,10 +148,10 @@ inline DistConst dist_const(double dmin, double dmax) {
 }
 
 #ifdef __CUDACC__
-// The distance marginal of log_distance_marginal with the same rules (48-point window of
-// +-12 widths about the peak, 4-panel 8-point composite rules outside it; 24 panels of 8
-// points without a peak), taken in FP32 about a reference point s_ref (the peak, or the
-// large-distance end): every node contributes G(s) - G(s_ref) from dist_rule_f, and G(s_ref)
+// The distance marginal (48-point window of +-12 widths about the peak, 4-panel 8-point composite
+// rules outside it; 24 panels of 8 points without a peak inside the range), taken in FP32 about a
+// reference point s_ref (the peak, the end of the range nearest to it, or the large-distance end):
+// every node contributes G(s) - G(s_ref) from dist_rule_f, and G(s_ref)
 // itself is assembled in FP64 from exact products,
 //   G(s_ref) = c0 - 3 s_ref + Z u_ref + [ln I0(Z u_ref) - Z u_ref] - H u_ref^2 / 2,
 // so that the few terms that grow with the signal (Z u_ref, H u_ref^2 reach 10^4) keep FP64

@@ -1,13 +1,15 @@
 // fixed.cuh -- fixed-point helpers of the double-precision kernels (host and device).
 //
 // The GB300 runs an FP64 instruction in 64 clocks per warp and SM quarter, a 32 x 32 + 64-bit
-// integer multiply-add in 4, a shift, an add or a logical operation in 2 (measured).  Quantities whose magnitude is bounded
-// -- a phase in turns, a sine or cosine, data scaled by their largest value -- therefore keep
-// FP64 accuracy and better as 64-bit integers split into two 28-bit halves,
-//   X = X1 2^28 + X0,  0 <= X0 < 2^28,
+// integer multiply-add in 4, a shift, an add or a logical operation in 2 (measured).  Quantities
+// whose magnitude is bounded -- a phase in turns, a sine or cosine, data scaled by their largest
+// value -- therefore keep FP64 accuracy and better as 64-bit integers split into two halves,
+//   X = X1 2^b + X0,
 // a product of which takes three multiply-adds:
-//   A B = A1 B1 2^56 + (A1 B0 + A0 B1) 2^28 + (A0 B0, dropped: 2^-56 of the result's scale).
-// "Unit 2^-56" below means a 64-bit integer holding the value times 2^56.
+//   A B = A1 B1 2^(2b) + (A1 B0 + A0 B1) 2^b + (A0 B0, dropped).
+// The FP64 likelihood takes balanced halves of b = 32 bits (Pair32 below), whose middle sum needs
+// no shift; draws, logarithms and exponentials take b = 28 with 0 <= X0 < 2^28 (Pair28).  "Unit
+// 2^-56" below means a 64-bit integer holding the value times 2^56.
 #pragma once
 #include <cstdint>
 #include <cstring>

@@ -25,7 +25,7 @@
 // While the tensor core runs block kb the threads compute block kb + 1's rows; then they add
 // block kb's accumulator into running sums kept in the other half of TMEM (FP32,
 // round-to-nearest), which frees the accumulator for block kb + 1.  The per-sample set-up
-// is split between the two threads of a sample (phase coefficients and cut on one, the
+// is split between two threads of a sample (phase coefficients and cut on one, the
 // detector responses and delays on the other) and exchanged through shared memory.  The A
 // operand never touches global memory; after the last block the running sums go through
 // shared memory (transposed) to the log-mean-exp.
@@ -175,7 +175,8 @@ __global__ void __launch_bounds__(kTT, kCtasPerSm) loglike_mixed_time_kernel(Lik
   const bool active = slot < a.n;
   const int64_t s = active && a.perm != nullptr ? (int64_t)a.perm[slot] : slot;
 
-  // ---- per-sample set-up (FP64), shared by the sample's two threads
+  // ---- per-sample set-up (float-float; FP64 for ln(pi M), the inputs and the cut), shared by the
+  // sample's first two threads
   double par[kNumSlots];
 #pragma unroll
   for (int i = 0; i < kNumSlots; ++i)

@@ -149,7 +149,7 @@ struct RbSmem {
   int32_t kcut[kRbTile];
   float part[2][kRbTile];            // the imaginary sum (hi, lo)
   float dist[6][kRbTile];            // the distance rule: lo, hi, Z, H, u_ref, phi_ref
-  int32_t nodes[kRbTile];            // its nodes: 48, 192 without a window, 0 outside the model
+  int32_t nodes[kRbTile];            // its shared nodes: 48, 192 without a window, 0 outside the model
   float g[2][kGL48][kRbTile];        // 48 node values at a time, two rounds in turn
 };
 
@@ -340,9 +340,9 @@ __global__ void __launch_bounds__(kRbThreads, 4) rb_loglike_kernel(RbArgs r) {
     sm.dist[3][si] = win.H;
     sm.dist[4][si] = win.u_ref;
     sm.dist[5][si] = win.phi_ref;
-    sm.nodes[si] = valid ? (win.window ? kGL48 : kDistFull) : 0;
+    sm.nodes[si] = valid ? dist_main_count(win) : 0;
   }
-  const bool any_full = __syncthreads_or(role == 0 && valid && !win.window);
+  const bool any_full = __syncthreads_or(role == 0 && sm.nodes[si] == kDistFull);
   LogSumExpF L;
   const int rounds = any_full ? kDistFull / kGL48 : 1;
   for (int rd = 0; rd < rounds; ++rd) {

@@ -192,19 +192,31 @@ __device__ __forceinline__ DistWindow dist_window(double Z, double H, const Dist
   return d;
 }
 
-// The main rule: 48 nodes over the window, or the whole range's without one.  node i: its offset
-// and expm1 of it.  The whole range's are tabled for the reference point at the large-distance
-// end, lo = 0; a peak beyond the near end puts the reference there (the growing terms then vanish
-// where the integrand is largest), and its nodes are evaluated.
+// The main rule: 48 nodes over the window; without one the whole range's, tabled for the reference
+// point at the large-distance end (lo = 0).  A peak beyond the near end puts the reference there,
+// where the integrand is largest and the growing terms vanish: no main rule then, dist_finish
+// evaluates the range.
+__device__ __forceinline__ int dist_main_count(const DistWindow& d) {
+  return d.window ? kGL48 : d.lo == 0.0f ? kDistFull : 0;
+}
+// node i: its offset and expm1 of it
 __device__ __forceinline__ float2 dist_main_node(bool window, float lo, float hi, const float* gl, int i) {
-  if (!window && lo == 0.0f) return make_float2(__ldg(gl + kGLSize + i), __ldg(gl + kGLSize + kDistFull + i));
-  const float d = window ? dist_node_at(lo, hi, 1, 0, __ldg(gl + i))
-                         : dist_node_at(lo, hi, 24, i / kGL8, __ldg(gl + 2 * kGL48 + i % kGL8));
+  if (!window) return make_float2(__ldg(gl + kGLSize + i), __ldg(gl + kGLSize + kDistFull + i));
+  const float d = dist_node_at(lo, hi, 1, 0, __ldg(gl + i));
   return make_float2(d, expm1f(d));
 }
 __device__ __forceinline__ float dist_main_weight(bool window, float lo, float hi, const float* gl, int i) {
   const float h = (hi - lo) * (window ? 1.0f : 1.0f / 24.0f);
   return 0.5f * h * __ldg(gl + (window ? kGL48 + i : 2 * kGL48 + kGL8 + i % kGL8));
+}
+
+// The whole range about the near end, for the rare source inside dmin: called, so that the kernels'
+// own code is that of the other two rules.
+static __device__ __noinline__ LogSumExpF dist_near_range(float lo, float hi, const float* x8, float Z, float H,
+                                                          float u_ref, float phi_ref) {
+  LogSumExpF L;
+  dist_rule_f(L, lo, hi, 24, kGL8, x8, x8 + kGL8, Z, H, u_ref, phi_ref);
+  return L;
 }
 
 // The marginal from the main rule's sum L.
@@ -226,6 +238,8 @@ __device__ __forceinline__ double dist_finish(const DistWindow& d, LogSumExpF L,
     }
     if (d.whi < dc.span && dist_node_g(d.hi, d.Z, d.H, d.u_ref, d.phi_ref) > L.m - kDistSkip)
       dist_rule_f(L, d.hi, dc.span - d.r_ref, 4, kGL8, x8, w8, d.Z, d.H, d.u_ref, d.phi_ref);
+  } else if (d.lo != 0.0f) {
+    L = dist_near_range(d.lo, d.hi, x8, d.Z, d.H, d.u_ref, d.phi_ref);
   }
   const double u_ref = to_double(d.u_ref);
   const double g_ref =
@@ -237,16 +251,15 @@ __device__ __forceinline__ double log_distance_marginal_mixed(double Z, double H
                                                               const float* gl) {
   const DistWindow d = dist_window(Z, H, dc);
   LogSumExpF L;
-  if (d.window)
+  if (d.window) {
     dist_rule_f(L, d.lo, d.hi, 1, kGL48, gl, gl + kGL48, d.Z, d.H, d.u_ref, d.phi_ref);
-  else
-    {
+  } else if (dist_main_count(d) > 0) {
 #pragma unroll 4
-      for (int i = 0; i < kDistFull; ++i) {
-        const float2 n = dist_main_node(false, d.lo, d.hi, gl, i);
-        L.add(dist_node_e(n.x, n.y, d.Z, d.H, d.u_ref, d.phi_ref), dist_main_weight(false, d.lo, d.hi, gl, i));
-      }
+    for (int i = 0; i < kDistFull; ++i) {
+      const float2 n = dist_main_node(false, d.lo, d.hi, gl, i);
+      L.add(dist_node_e(n.x, n.y, d.Z, d.H, d.u_ref, d.phi_ref), dist_main_weight(false, d.lo, d.hi, gl, i));
     }
+  }
   return dist_finish(d, L, Z, H, dc, gl);
 }
 #endif

@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawCons
     }
   }
   double mc = 0.0, q = 0.0;
-  bool inside = true, polar = false;
+  bool inside = true;
   int64_t log_sum51 = 0, polar53 = 0;  // the prior's logarithms, units 2^-51 and 2^-53
 #pragma unroll
   for (int p = 0; p < P; ++p) {
@@ -209,21 +209,21 @@ __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawCons
       // poles: within kPolar of one, ln d + ln(sin d / d) of the angle d from it
       const double y = !inside ? 1.0 : id == kDec ? fabs(x) : x, pole = id == kDec ? 0.5 * kPi : kPi;
       const bool face_on = id == kIota && order_key(y) < order_key(kPolar);
-      int64_t v;
+      LogArg arg;
+      int64_t sinc = 0;
       if (face_on || order_key(y) > order_key(pole - kPolar)) {
         const double d = face_on ? y : (pole - y) + (id == kDec ? 0.5 * kPiTail : kPiTail);
-        const LogArg arg = log_arg(d);
-        v = log_sum(arg.e, log_mantissa(tb, arg.m) + log_sinc(d));
+        arg = log_arg(d);
+        sinc = log_sinc(d);
         if (order_key(d) == 0) inside = false;  // at the pole: ln 0
       } else {
         int64_t co, si;
         trig_of(tb, angle_turns(y), co, si);
         const uint64_t w = (uint64_t)(id == kDec ? co : si);
         const int lz = clz64(w);
-        v = log_sum(1 - lz, log_mantissa(tb, w << lz));
+        arg = LogArg{w << lz, 1 - lz};
       }
-      polar53 += v;
-      polar = true;
+      polar53 += log_sum(arg.e, log_mantissa(tb, arg.m) + sinc);
     }
     if (id == kDl) log_sum51 += (log_of(tb, inside ? x : 1.0) + 1) >> 1;
   }
@@ -241,8 +241,11 @@ __global__ void __launch_bounds__(kDrawThreads) draw_kernel(DrawArgs a, DrawCons
                   __mul64hi(lq, 0x3333333333333333ll) + 2) >> 2;
   }
   if (a.logp) {
-    if (polar) lp = fma((double)polar53, 0x1p-53, k.lp_const);
-    a.logp[i] = inside ? fma((double)log_sum51, 0x1p-51, polar ? lp : k.lp_const) : -INFINITY;
+    // one sum in unit 2^-53 where it holds both (|ln cos dec + ln sin iota| < 800)
+    const bool both = log_sum51 < (1ll << 58) && log_sum51 > -(1ll << 58);
+    lp = fma((double)(both ? polar53 + log_sum51 * 4 : polar53), 0x1p-53, k.lp_const);
+    if (!both) lp = fma((double)log_sum51, 0x1p-51, lp);
+    a.logp[i] = inside ? lp : -INFINITY;
   }
   if (a.logq) a.logq[i] = a.log_q_const - half_zz;
 }

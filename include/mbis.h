@@ -148,7 +148,8 @@ mbis_status mbis_loglike(mbis_ctx* ctx, int64_t n, const double* theta, double* 
 
 /* Importance weights and Kish ESS (Eqs. 5-6), evidence Z = mean(w):
  * m = max(log L + log pi - log g), then FP64 sums S1 = sum e^(log w - m),
- * S2 = sum e^(2 (log w - m)), in one pass on the device (sums about each CTA's own maximum).  Inputs (device, n each).  weights_out (device, n) gets the
+ * S2 = sum e^(2 (log w - m)), in one pass on the device (sums about each CTA's own maximum).
+ * Inputs (device, n each).  weights_out (device, n; it may be one of the inputs) gets the
  * normalised weights e^(log w - m) / S1 when not NULL.  accumulate != 0 merges this batch
  * into the context's running state and reports the merged summary; 0 reports this batch
  * alone and leaves the running state untouched.  *out (host) receives the summary;

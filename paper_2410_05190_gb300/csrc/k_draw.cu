@@ -20,8 +20,8 @@
 //     batches), and a refit feeds such a difference back: with this choice a seed keeps its
 //     results.  (The sum of squares takes explicit multiply-adds: an unrolled chain of sums is
 //     re-associated when it is contracted.)
-// Measured on a GB300 (device time): 2^18 samples of 11 slots 429 us before and 58 us fixed;
-// 2^16 of 5 slots 50 us before, 10 us fixed.
+// Measured on a GB300 (device time): 2^18 samples of 11 slots 429 us before and 61 us fixed;
+// 2^16 of 5 slots 50 us before, 12 us fixed.
 #include <algorithm>
 #include <cmath>
 

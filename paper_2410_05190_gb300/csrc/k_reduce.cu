@@ -13,8 +13,8 @@
 // some 30 instructions), the maxima on the integer pipe, and a warp's two sums fold with five
 // adds between them, which leaves five FP64 instructions per sample.  Measured on a GB300 with
 // weights (device time): 94 us at 2^18 samples, 78 at 2^16 and 74 at 4096 for the three launches
-// of the first version (its sum ended in one thread adding 608 partials), 28, 17 and 15
-// here.
+// of the first version (its sum ended in one thread adding 608 partials), 29 (22 and 6), 17 and
+// 14 here.
 #include <algorithm>
 
 #include "fixed.cuh"
